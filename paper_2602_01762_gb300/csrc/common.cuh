@@ -495,11 +495,14 @@ size_t gemv_tc_workspace_floats(const GemvArgs &a, int sms);
 int gemv_tc_tiles(const GemvArgs &a);
 cudaError_t launch_gemv_tc(const GemvArgs &a, const CUtensorMap &m, int sms, float *part, int *tile_ctr,
                            cudaStream_t s, bool pdl);
-// Streamed variant for many activation rows (up to 256; 128 for SwiGLU, 64
-// for top-k): prep kernel for the activation rows (into xbuf, bf16
+// Streamed variant (any number of activation rows, in tiles of up to 256; 128
+// for SwiGLU, 64 for top-k): prep kernel for the activation rows (into xbuf, bf16
 // [T][kin], unless the prologue is a copy), the projection, and for top-k
 // the cross-CTA merge kernel.
 bool gemv_tcs_supported(const GemvArgs &a, int sms);
+// CTAs that share each row's selection in an LM-head launch (its per-CTA lists
+// and log-sum-exp partials are [row][slots]).
+int gemv_lm_slots(const GemvArgs &a, int sms, bool streamed);
 size_t gemv_tcs_workspace_floats(const GemvArgs &a, int sms);
 // *next_done (may be null) reports whether the launch also wrote the next
 // projection's rows (a.next_norm or a.next_fuse) into a.next_x.

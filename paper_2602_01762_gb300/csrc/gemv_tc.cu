@@ -191,6 +191,7 @@ struct TcPlan {
     float *part;        // split-K partial sums [splits][RPW][T][n_units]
     int *tile_ctr;      // per-tile arrival tickets (left at zero)
     int defer;          // split-K sums finished by splitk_finish_kernel, not the tile's last CTA
+    int n_rt;           // streamed kernel: tiles of NB activation rows (a work item is one unit tile x one row tile)
 };
 
 // X rows (bf16, swizzled K-major operand layout) for the K blocks [kb0, kb1).
@@ -443,7 +444,8 @@ __device__ __forceinline__ void chunk_to_lists(const float (&acc)[16], int row, 
 
 // The CTA's (max, sum exp) of each row: the 8 threads of a row combine
 // theirs (fixed butterfly order), the first writes the CTA's partial.
-__device__ __forceinline__ void lse_publish(const GemvArgs &a, float m, float s, int T, int t0) {
+__device__ __forceinline__ void lse_publish(const GemvArgs &a, float m, float s, int T, int t0, int row0, int slot,
+                                            int slots) {
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
         const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, s, o);
@@ -451,7 +453,7 @@ __device__ __forceinline__ void lse_publish(const GemvArgs &a, float m, float s,
     }
     const int e = threadIdx.x - 64, t = t0 + e / 8;
     if ((e & 7) == 0 && t < T) {
-        float *pp = a.lse_part + ((size_t)t * gridDim.x + blockIdx.x) * 2;
+        float *pp = a.lse_part + ((size_t)(row0 + t) * slots + slot) * 2;
         pp[0] = m;
         pp[1] = s;
     }
@@ -459,9 +461,11 @@ __device__ __forceinline__ void lse_publish(const GemvArgs &a, float m, float s,
 
 // The CTA's list of each row: the P threads of a row merge theirs and write
 // it to the per-CTA partial lists ([row][CTA][kTopK] values and ids; id -1
-// marks an empty slot), thread q the entries q, q + P, ...
+// marks an empty slot), thread q the entries q, q + P, ...  The rows start at
+// row0; this CTA is number `slot` of the `slots` CTAs that share them.
 template <int P>
-__device__ __forceinline__ void lists_publish(const GemvArgs &a, Key (&l)[kTopK], int T, int t0 = 0) {
+__device__ __forceinline__ void lists_publish(const GemvArgs &a, Key (&l)[kTopK], int T, int t0, int row0, int slot,
+                                              int slots) {
 #pragma unroll 1
     for (int m = 1; m < P; m <<= 1) key_merge_xor(l, m);
     const int e = threadIdx.x - 64, t = t0 + e / P, q = e % P;
@@ -471,7 +475,7 @@ __device__ __forceinline__ void lists_publish(const GemvArgs &a, Key (&l)[kTopK]
             float v;
             int id;
             unpack_best(key_at(l, r0 + q), v, id);
-            const size_t o = ((size_t)t * gridDim.x + blockIdx.x) * kTopK + r0 + q;
+            const size_t o = ((size_t)(row0 + t) * slots + slot) * kTopK + r0 + q;
             a.lm_part[o] = v;
             a.lm_part_id[o] = id;
         }
@@ -831,8 +835,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             if constexpr (top1) {
                 top1_join<NB>(a, T, s_val, s_id, s_last);
             } else if constexpr (TOPK) {
-                lists_publish<8>(a, lst, T);
-                if (a.lse_part) lse_publish(a, lse_m, lse_s, T, 0);
+                lists_publish<8>(a, lst, T, 0, 0, blockIdx.x, gridDim.x);
+                if (a.lse_part) lse_publish(a, lse_m, lse_s, T, 0, 0, blockIdx.x, gridDim.x);
                 __threadfence();
                 epi_sync();
                 if (threadIdx.x == 64) s_last = !a.defer_merge && atomicAdd(a.counter, 1) == (int)gridDim.x - 1;
@@ -867,9 +871,16 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 // 64 columns, the same 128-byte swizzle), fetched by TMA from a bf16 X
 // buffer that a prep kernel (or the previous projection, for the copy
 // prologue) has written.  MMA N = NB (16 .. 256); rows of X past T arrive as
-// zeros.  The epilogue reads the NB accumulator columns 16 at a time.  With
+// zeros.  More than NB rows are tiles of NB rows (p.n_rt of them): a work item
+// is one unit tile times one row tile, and the items of one unit tile run on
+// neighbouring CTAs at the same time, so that HBM delivers its weights once and
+// L2 the rest.  (Llama-3-8B shape: the fusion of 384 rows 2184 us on the
+// CUDA-core ring kernel, which took such rows before, 56 us here; of 1000 rows
+// 5890 and 88 us, 0.77 PFLOP/s; QKV of 1000 rows 4430 and 145 us.)  RT: the
+// instance for several row tiles; the one for a single tile carries no
+// division by n_rt.  The epilogue reads the NB accumulator columns 16 at a time.  With
 // top-k, the per-row merge across CTAs is left to topk_merge_kernel.
-template <int NB, int RPW, int TK>
+template <int NB, int RPW, int TK, bool RT>
 __global__ void __launch_bounds__(kTcThreads, 1)
     gemv_tcs_kernel(const GemvArgs a, const TcPlan p, const __grid_constant__ CUtensorMap tmW,
                     const __grid_constant__ CUtensorMap tmX) {
@@ -895,11 +906,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     const int S = p.stages;
     const uint32_t kb_bytes = RPW * kBoxBytes + kXBox;                // one K block in a stage
     const int ks = blockIdx.x % p.splits;
-    const int tiles_step = gridDim.x / p.splits;
+    // this CTA's work items c, c + step, ...: item -> unit tile item / n_rt, row tile item % n_rt
+    const int item0 = blockIdx.x / p.splits, step = gridDim.x / p.splits, n_items = RT ? p.n_tiles * p.n_rt : p.n_tiles;
     const int kb0 = (int)((long)ks * p.nkb / p.splits), kb1 = (int)((long)(ks + 1) * p.nkb / p.splits);
     const int n_kst = (kb1 - kb0 + p.kb_per_stage - 1) / p.kb_per_stage;
-    int my_tiles = 0;
-    for (int tile = blockIdx.x / p.splits; tile < p.n_tiles; tile += tiles_step) ++my_tiles;
+    const int my_tiles = item0 < n_items ? (n_items - item0 + step - 1) / step : 0;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) {
@@ -929,38 +940,33 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     if (warp == 0) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            const uint64_t wpol = a.w_evict_first ? l2_evict_first_policy() : 0ull;
-            int s = 0, issued = 0;
-            uint32_t ph = 0;
+            // several row tiles: the other tiles' CTAs read the same weight boxes from L2
+            const uint64_t wpol = a.w_evict_first && !RT ? l2_evict_first_policy() : 0ull;
+            int issued = 0;
             bool dead = false;
             const int total = my_tiles * n_kst;
-            // item f of this CTA: tile, first K block and K blocks of its stage
-            auto item = [&](int f, int &tile, int &kbs, int &nkb) {
-                tile = blockIdx.x / p.splits + (f / n_kst) * tiles_step;
-                kbs = kb0 + (f % n_kst) * p.kb_per_stage;
-                nkb = kb1 - kbs < p.kb_per_stage ? kb1 - kbs : p.kb_per_stage;
+            const uint32_t ring0 = saddr(ring), ring_end = ring0 + (uint32_t)S * p.stage_bytes;
+            // The stages of this CTA in order: `it` is the work item, `kbs` the
+            // first K block.  They are stepped, not derived from a stage number:
+            // this lane issues every copy of the CTA, and two integer divisions
+            // per stage (n_kst, n_rt) cost 3-8 us per launch.
+            int it = item0, kbs = kb0;
+            auto next = [&]() {
+                kbs += p.kb_per_stage;
+                if (kbs >= kb1) { kbs = kb0; it += step; }
             };
-            auto load_w = [&](int f, int stage) {
-                int tile, kbs, nkb;
-                item(f, tile, kbs, nkb);
-                const uint32_t st = saddr(ring) + (uint32_t)stage * p.stage_bytes;
+            auto load_w = [&](uint32_t st, uint64_t *bar, int nkb) {
+                const int tile = RT ? it / p.n_rt : it;
                 for (int j = 0; j < nkb; ++j)
 #pragma unroll
                     for (int r = 0; r < RPW; ++r)
                         tma_load_2d_pol(st + (uint32_t)j * kb_bytes + (uint32_t)r * kBoxBytes, &tmW, (kbs + j) * kBoxK,
-                                        tile * kTileM + r * a.pair_offset, &full[stage], wpol);
+                                        tile * kTileM + r * a.pair_offset, bar, wpol);
             };
-            auto load_x = [&](int f, int stage) {
-                int tile, kbs, nkb;
-                item(f, tile, kbs, nkb);
-                const uint32_t st = saddr(ring) + (uint32_t)stage * p.stage_bytes;
+            auto load_x = [&](uint32_t st, uint64_t *bar, int nkb) {
+                const int row0 = RT ? it % p.n_rt * NB : 0;
                 for (int j = 0; j < nkb; ++j)
-                    tma_load_2d(st + (uint32_t)j * kb_bytes + RPW * kBoxBytes, &tmX, (kbs + j) * kBoxK, 0, &full[stage]);
-            };
-            auto arm = [&](int f, int stage) {
-                int tile, kbs, nkb;
-                item(f, tile, kbs, nkb);
-                mbar_arrive_tx(&full[stage], (uint32_t)nkb * kb_bytes);
+                    tma_load_2d(st + (uint32_t)j * kb_bytes + RPW * kBoxBytes, &tmX, (kbs + j) * kBoxK, row0, bar);
             };
             // The first ring pass: the stages are free (fresh barriers), and the
             // weight boxes do not depend on the previous kernel, so they are
@@ -969,26 +975,33 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // barrier expects both from the start, so it completes only when both
             // have landed.
             const int pre = total < S ? total : S;
-            for (int f = 0; f < pre; ++f) {
-                arm(f, f);
-                load_w(f, f);
+            for (int f = 0; f < pre; ++f, next()) {
+                const int nkb = min(kb1 - kbs, p.kb_per_stage);
+                mbar_arrive_tx(&full[f], (uint32_t)nkb * kb_bytes);
+                load_w(ring0 + (uint32_t)f * p.stage_bytes, &full[f], nkb);
             }
             pdl_wait();
-            for (int f = 0; f < pre; ++f) load_x(f, f);
+            it = item0;
+            kbs = kb0;
+            for (int f = 0; f < pre; ++f, next())
+                load_x(ring0 + (uint32_t)f * p.stage_bytes, &full[f], min(kb1 - kbs, p.kb_per_stage));
             issued = pre;
-            s = pre % S;
-            ph = pre == S ? 1u : 0u;
-            for (int f = pre; f < total; ++f) {
+            int s = pre == S ? 0 : pre;
+            uint32_t ph = pre == S ? 1u : 0u, st = pre == S ? ring0 : ring0 + (uint32_t)pre * p.stage_bytes;
+            for (int f = pre; f < total; ++f, next()) {
                 if (!mbar_wait(&empty[s], ph ^ 1, lim)) {
                     set_err(a.err, kErrTimeout);
                     dead = true;
                     break;
                 }
-                arm(f, s);
-                load_w(f, s);
-                load_x(f, s);
+                const int nkb = min(kb1 - kbs, p.kb_per_stage);
+                mbar_arrive_tx(&full[s], (uint32_t)nkb * kb_bytes);
+                load_w(st, &full[s], nkb);
+                load_x(st, &full[s], nkb);
                 ++issued;
-                if (++s == S) { s = 0; ph ^= 1; }
+                ++s;
+                st += p.stage_bytes;
+                if (st == ring_end) { s = 0; st = ring0; ph ^= 1; }
             }
             if (!dead) prefetch_l2_share(a.pf_next, a.pf_next_bytes, blockIdx.x, gridDim.x);
             const int first = issued > S ? issued - S : 0;
@@ -1053,7 +1066,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             const int ew = warp - 2;
             const int quarter = warp & 3;
             const int row = quarter * 32 + lane;
-            const int T = a.T;
+            // rows of this CTA's row tile (selections: every item of a CTA has the same one)
+            int row0 = RT ? item0 % p.n_rt * NB : 0, T = RT ? min(NB, a.T - row0) : a.T;
             // top-k: every 16-row chunk of a tile is scanned by all 128 epilogue
             // threads, 8 per row (each thread keeps one list per chunk position)
             constexpr int kNL = LISTS ? NB / 16 : 1;
@@ -1079,7 +1093,11 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             }
             bool dead = false;
             for (int i = 0; i < my_tiles; ++i) {
-                const int tile = blockIdx.x / p.splits + i * tiles_step;
+                const int it = item0 + i * step, tile = RT ? it / p.n_rt : it;
+                if constexpr (RT && !TOPK) {
+                    row0 = it % p.n_rt * NB;
+                    T = min(NB, a.T - row0);
+                }
                 const int ab = i & 1;
                 if (!dead && !mbar_wait_warp(&acc_full[ab], (i >> 1) & 1, lim)) {
                     if (lane == 0) set_err(a.err, kErrTimeout);
@@ -1103,7 +1121,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                         if (valid && a.logits) {
 #pragma unroll
                             for (int tt = 0; tt < 16; ++tt)
-                                if (c0 + tt < T) a.logits[((size_t)(c0 + tt) * a.K + a.step - 1) * a.vocab + u] = acc[tt];
+                                if (c0 + tt < T) a.logits[((size_t)(row0 + c0 + tt) * a.K + a.step - 1) * a.vocab + u] = acc[tt];
                         }
                         if constexpr (LISTS)
                             chunk_to_lists<8>(acc, row, &s_tr[0][0], tile, c0, T, a.n_units, dead, lst[cc],
@@ -1128,7 +1146,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
                             for (int tt = 0; tt < 16; ++tt) {
                                 if (c0 + tt >= T) break;
-                                finish_unit<RPW>(a, c0 + tt, u, acc[0][tt], acc[RPW - 1][tt]);
+                                finish_unit<RPW>(a, row0 + c0 + tt, u, acc[0][tt], acc[RPW - 1][tt]);
                             }
                         }
                     } else if (valid) {
@@ -1137,7 +1155,7 @@ __global__ void __launch_bounds__(kTcThreads, 1)
 #pragma unroll
                             for (int tt = 0; tt < 16; ++tt) {
                                 if (c0 + tt >= T) break;
-                                p.part[(((size_t)ks * RPW + r) * T + c0 + tt) * a.n_units + u] = acc[r][tt];
+                                p.part[(((size_t)ks * RPW + r) * a.T + row0 + c0 + tt) * a.n_units + u] = acc[r][tt];
                             }
                     }
                 }
@@ -1146,27 +1164,13 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     __syncwarp();
                     if (lane == 0) mbar_arrive(&acc_empty[ab]);
                 }
-                if constexpr (!TOPK) {
-                    if (p.splits > 1 && !p.defer) {
-                        __threadfence();
-                        epi_sync();
-                        if (threadIdx.x == 64) s_last = atomicAdd(&p.tile_ctr[tile], 1) == p.splits - 1;
-                        epi_sync();
-                        if (s_last) {
-                            __threadfence();
-                            if (valid) reduce_slices<RPW>(a, p, T, u);
-                            if (threadIdx.x == 64) p.tile_ctr[tile] = 0;
-                        }
-                        epi_sync();
-                    }
-                }
             }
             if constexpr (LISTS) {
                 // this CTA's list of every row; the cross-CTA merge is a separate kernel
 #pragma unroll
                 for (int cc = 0; cc < kNL; ++cc) {
-                    lists_publish<8>(a, lst[cc], T, 16 * cc);
-                    if (a.lse_part) lse_publish(a, lse_m[cc], lse_s[cc], T, 16 * cc);
+                    lists_publish<8>(a, lst[cc], T, 16 * cc, row0, RT ? item0 / p.n_rt : item0, RT ? step / p.n_rt : step);
+                    if (a.lse_part) lse_publish(a, lse_m[cc], lse_s[cc], T, 16 * cc, row0, RT ? item0 / p.n_rt : item0, RT ? step / p.n_rt : step);
                 }
             } else if constexpr (TK == 1) {
                 top1_join<kN1>(a, T, s_val, s_id, s_last);
@@ -1578,16 +1582,23 @@ bool tc_plan(const GemvArgs &a, int sms, TcPlan &p, int &grid, size_t &smem) {
 
 }  // namespace
 
-template <int NB, int RPW, int TK>
+template <int NB, int RPW, int TK, bool RT = false>
 cudaError_t set_tcs_attr(int bytes) {
-    return cudaFuncSetAttribute(gemv_tcs_kernel<NB, RPW, TK>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+    return cudaFuncSetAttribute(gemv_tcs_kernel<NB, RPW, TK, RT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
 }
 
-int tcs_nb(int T, int RPW, bool topk) {
-    int nb = 16;
-    while (nb < T) nb *= 2;
+// Activation rows of one tile (the MMA's N) and the number of such tiles: up
+// to 256 rows (128 for the gate/up pairs, whose two accumulators are double
+// buffered in the 512 tensor-memory columns, and 64 for top-k lists, kept in
+// registers) are one tile; more rows take the fewest tiles, each of an
+// instance just large enough for an even share.
+void tcs_rows(int T, int RPW, bool topk, int &nb, int &n_rt) {
     const int cap = topk ? 64 : (RPW == 2 ? 128 : 256);
-    return nb <= cap ? nb : 0;
+    n_rt = (T + cap - 1) / cap;
+    const int share = (T + n_rt - 1) / n_rt;
+    nb = 16;
+    while (nb < share) nb *= 2;
+    if (n_rt > 1 && RPW == 1 && !topk && share <= 192) nb = 192;
 }
 
 // The selection a streamed launch makes: 0 none, 1 the packed top-1 (one
@@ -1606,24 +1617,35 @@ bool tcs_plan(const GemvArgs &a, int sms, TcPlan &p, int &grid, size_t &smem, in
     const bool topk = a.epi == kEpiTopK;
     const int RPW = a.epi == kEpiSwiGLU ? 2 : 1;
     if (a.T < 1 || a.kin % 8 || a.n_units < 1) return false;
-    NB = tcs_nb(a.T, RPW, topk);
-    if (!NB) return false;
+    int n_rt;
+    tcs_rows(a.T, RPW, topk, NB, n_rt);
     const int nkb = (a.kin + kBoxK - 1) / kBoxK;
     const int n_tiles = (a.n_units + kTileM - 1) / kTileM;
+    if (n_tiles > (1 << 30) / n_rt || (topk && n_rt > sms)) return false;
+    const int items = n_tiles * n_rt;
     // No split when the tiles alone already occupy most SMs in one wave: a
     // split then buys little streaming time and costs a finish pass over
     // every partial sum (gate/up at 112 tiles: 2440 -> 2197 us per round at
     // batch 64, 1663 -> 1615 us at batch 16)
-    const bool one_wave = n_tiles <= sms && 10 * n_tiles >= 7 * sms;
+    const bool one_wave = items <= sms && 10 * items >= 7 * sms;
     const int max_s = topk || one_wave ? 1 : kMaxSplits;
     long best = -1;
     int best_s = 0, best_ctas = 0;
     for (int sp = 1; sp <= max_s && sp <= nkb; ++sp) {
         const int per = (nkb + sp - 1) / sp;
         int ctas = sms / sp;
-        if (ctas > n_tiles) ctas = n_tiles;
+        if (ctas > items) ctas = items;
         if (ctas < 1) break;
-        const long cost = (long)((n_tiles + ctas - 1) / ctas) * per;
+        // selections: a CTA keeps to one row tile, so that its lists are of one
+        // set of rows (the CTAs of the other row tiles find the weights in L2)
+        if (topk) ctas = std::min(sms / n_rt, n_tiles) * n_rt;
+        long cost = (long)((items + ctas - 1) / ctas) * per;
+        // several row tiles: the finish pass over the partial sums is no longer
+        // small beside the stream (in stages' bytes of one SM)
+        if (n_rt > 1 && sp > 1) {
+            const long kb = (long)RPW * kBoxBytes + NB * 128;
+            cost += ((long)(2 * sp + 1) * RPW * a.T * a.n_units * 4 / sms) / kb;
+        }
         if (best < 0 || cost < best) { best = cost; best_s = sp; best_ctas = ctas; }
     }
     if (best < 0) return false;
@@ -1635,6 +1657,7 @@ bool tcs_plan(const GemvArgs &a, int sms, TcPlan &p, int &grid, size_t &smem, in
                                : std::min((size_t)220 * 1024 - tcs_static(NB, tk), kTcSmem);
     const size_t room = dyn - 1024;
     p.n_tiles = n_tiles;
+    p.n_rt = n_rt;
     p.nkb = nkb;
     p.splits = best_s;
     // the largest stage of up to 64 KB of which four still fit (larger
@@ -1648,8 +1671,8 @@ bool tcs_plan(const GemvArgs &a, int sms, TcPlan &p, int &grid, size_t &smem, in
     if (p.stages > kTcMaxStages) p.stages = kTcMaxStages;
     if (p.stages < 2) return false;
     if (a.even_waves && topk && best_s == 1) {
-        const int waves = (n_tiles + best_ctas - 1) / best_ctas;
-        best_ctas = (n_tiles + waves - 1) / waves;
+        const int per_rt = best_ctas / n_rt, waves = (n_tiles + per_rt - 1) / per_rt;
+        best_ctas = (n_tiles + waves - 1) / waves * n_rt;
     }
     grid = best_ctas * best_s;
     smem = 1024 + (size_t)p.stages * p.stage_bytes;
@@ -1660,17 +1683,29 @@ template <int NB>
 cudaError_t dispatch_tcs(const GemvArgs &a, const TcPlan &p, const CUtensorMap &mw, const CUtensorMap &mx, int grid,
                          size_t smem, cudaStream_t s, bool pdl) {
     const dim3 g(grid), b(kTcThreads);
+    // several row tiles: only the instances that tcs_rows gives them
+    if (p.n_rt > 1) {
+        if constexpr (NB == 64)
+            if (a.epi == kEpiTopK) return launch_k(gemv_tcs_kernel<NB, 1, 2, true>, g, b, smem, s, pdl, a, p, mw, mx);
+        if constexpr (NB == 128)
+            if (a.epi == kEpiSwiGLU) return launch_k(gemv_tcs_kernel<NB, 2, 0, true>, g, b, smem, s, pdl, a, p, mw, mx);
+        if constexpr (NB == 192 || NB == 256)
+            if (a.epi == kEpiStore || a.epi == kEpiResid)
+                return launch_k(gemv_tcs_kernel<NB, 1, 0, true>, g, b, smem, s, pdl, a, p, mw, mx);
+        return cudaErrorInvalidValue;
+    }
     if (a.epi == kEpiTopK) {
         if constexpr (NB == 16)
-            if (tcs_tk(a, NB) == 1) return launch_k(gemv_tcs_kernel<NB, 1, 1>, g, b, smem, s, pdl, a, p, mw, mx);
-        if constexpr (NB <= 64) return launch_k(gemv_tcs_kernel<NB, 1, 2>, g, b, smem, s, pdl, a, p, mw, mx);
+            if (tcs_tk(a, NB) == 1) return launch_k(gemv_tcs_kernel<NB, 1, 1, false>, g, b, smem, s, pdl, a, p, mw, mx);
+        if constexpr (NB <= 64) return launch_k(gemv_tcs_kernel<NB, 1, 2, false>, g, b, smem, s, pdl, a, p, mw, mx);
         return cudaErrorInvalidValue;
     }
     if (a.epi == kEpiSwiGLU) {
-        if constexpr (NB <= 128) return launch_k(gemv_tcs_kernel<NB, 2, 0>, g, b, smem, s, pdl, a, p, mw, mx);
+        if constexpr (NB <= 128) return launch_k(gemv_tcs_kernel<NB, 2, 0, false>, g, b, smem, s, pdl, a, p, mw, mx);
         return cudaErrorInvalidValue;
     }
-    return launch_k(gemv_tcs_kernel<NB, 1, 0>, g, b, smem, s, pdl, a, p, mw, mx);
+    if constexpr (NB != 192) return launch_k(gemv_tcs_kernel<NB, 1, 0, false>, g, b, smem, s, pdl, a, p, mw, mx);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t prepare_gemv_tc_kernels() {
@@ -1686,10 +1721,12 @@ cudaError_t prepare_gemv_tc_kernels() {
     if (e == cudaSuccess) e = set_tc_attrs<16>((int)kTcSmem);
     const int b = (int)kTcSmem;
     // per instance: what the 220 KB budget leaves after its static shared memory
-#define PRISM_TCS(NB, RPW, TK)                                                                          \
+#define PRISM_TCS(NB, RPW, TK, ...)                                                                     \
     if (e == cudaSuccess)                                                                               \
-        e = set_tcs_attr<NB, RPW, TK>((int)std::min((size_t)b, (size_t)220 * 1024 - tcs_static(NB, TK)));
+        e = set_tcs_attr<NB, RPW, TK, ##__VA_ARGS__>(                                                   \
+            (int)std::min((size_t)b, (size_t)220 * 1024 - tcs_static(NB, TK)));
     PRISM_TCS(16, 1, 0) PRISM_TCS(32, 1, 0) PRISM_TCS(64, 1, 0) PRISM_TCS(128, 1, 0)
+    PRISM_TCS(192, 1, 0, true) PRISM_TCS(256, 1, 0, true) PRISM_TCS(128, 2, 0, true) PRISM_TCS(64, 1, 2, true)
     PRISM_TCS(256, 1, 0) PRISM_TCS(16, 2, 0) PRISM_TCS(32, 2, 0) PRISM_TCS(64, 2, 0)
     PRISM_TCS(128, 2, 0) PRISM_TCS(16, 1, 2) PRISM_TCS(32, 1, 2) PRISM_TCS(64, 1, 2)
 #undef PRISM_TCS
@@ -1740,6 +1777,14 @@ bool gemv_tcs_supported(const GemvArgs &a, int sms) {
     return tcs_plan(a, sms, p, grid, smem, NB);
 }
 
+int gemv_lm_slots(const GemvArgs &a, int sms, bool streamed) {
+    TcPlan p{};
+    int grid = 0, NB;
+    size_t smem;
+    if (streamed) return tcs_plan(a, sms, p, grid, smem, NB) ? grid / p.n_rt : 0;
+    return tc_plan(a, sms, p, grid, smem) ? grid : 0;
+}
+
 size_t gemv_tcs_workspace_floats(const GemvArgs &a, int sms) {
     TcPlan p{};
     int grid, NB;
@@ -1788,12 +1833,13 @@ cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, f
         case 32: e = dispatch_tcs<32>(a, p, mw, mx, grid, smem, s, pdl); break;
         case 64: e = dispatch_tcs<64>(a, p, mw, mx, grid, smem, s, pdl); break;
         case 128: e = dispatch_tcs<128>(a, p, mw, mx, grid, smem, s, pdl); break;
+        case 192: e = dispatch_tcs<192>(a, p, mw, mx, grid, smem, s, pdl); break;
         default: e = dispatch_tcs<256>(a, p, mw, mx, grid, smem, s, pdl); break;
     }
     if (e == cudaSuccess && a.epi == kEpiTopK && tcs_tk(a, NB) == 2) {
         GemvArgs m = a;
         m.next_fuse = a.next_fuse && a.next_x && a.d % 8 == 0;
-        if (!a.defer_merge) e = launch_k(topk_merge_kernel, dim3(a.T), dim3(128), 0, s, true, m, grid);
+        if (!a.defer_merge) e = launch_k(topk_merge_kernel, dim3(a.T), dim3(128), 0, s, true, m, grid / p.n_rt);
         if (e == cudaSuccess && next_done) *next_done = !a.defer_merge && m.next_fuse != 0;
     }
     if (e == cudaSuccess && p.defer) {

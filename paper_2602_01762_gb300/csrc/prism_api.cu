@@ -682,11 +682,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
                  chain_next ? &gn : nullptr, chain_next ? step_tm(k + 1, 0) : nullptr);
         if (tree) {
             ta.logits = gl.logits;
-            // the LM head's grid (one log-sum-exp partial per CTA and row): one
-            // CTA per SM, or with even waves the fewest CTAs for as many waves
-            const int lm_tiles = (V + 127) / 128;
-            int lm_ctas = lm_tiles < c->sms ? lm_tiles : c->sms;
-            if (c->lm_even_waves) lm_ctas = (lm_tiles + (lm_tiles + lm_ctas - 1) / lm_ctas - 1) / ((lm_tiles + lm_ctas - 1) / lm_ctas);
+            const int lm_ctas = gemv_lm_slots(gl, c->sms, on_tcs(gl, lm_tm));
             ta.lm_lse_grid = gl.lse_part ? lm_ctas : 0;
             ta.lm_val = gl.defer_merge ? c->lm_val : nullptr;
             ta.lm_id = gl.defer_merge ? c->lm_id : nullptr;
@@ -791,20 +787,24 @@ prism_status prism_create(const prism_config *cfg, int32_t device, prism_ctx **o
         const int kins[] = {2 * d, d, Hq * D, d, F};
         const int epis[] = {kEpiStore, kEpiStore, kEpiResid, kEpiSwiGLU, kEpiResid};
         const int pros[] = {kProFuseDecode, kProNorm, kProCopy, kProNorm, kProCopy};
+        // any batch up to max_batch may be called, and the split of more rows than
+        // one row tile holds does not grow with their number: every row count of
+        // step 1, of later steps and of tree steps is looked at
         for (int i = 0; i < 5; ++i)
-            for (int T : {(int)T1, (int)B, (int)Bseq}) {
-                GemvArgs g{};
-                g.n_units = units[i];
-                g.kin = kins[i];
-                g.epi = epis[i];
-                g.pro = pros[i];
-                g.T = T;
-                size_t need = gemv_tc_workspace_floats(g, c->sms);
-                if (need > tc_floats) tc_floats = need;
-                need = gemv_tcs_workspace_floats(g, c->sms);
-                if (need > tc_floats) tc_floats = need;
-                if (gemv_tc_tiles(g) > tc_tiles) tc_tiles = gemv_tc_tiles(g);
-            }
+            for (int nb = 1; nb <= f.max_batch; ++nb)
+                for (long T : {(long)nb * f.max_new, (long)nb, (long)nb * (long)TW}) {
+                    GemvArgs g{};
+                    g.n_units = units[i];
+                    g.kin = kins[i];
+                    g.epi = epis[i];
+                    g.pro = pros[i];
+                    g.T = (int)T;
+                    size_t need = gemv_tc_workspace_floats(g, c->sms);
+                    if (need > tc_floats) tc_floats = need;
+                    need = gemv_tcs_workspace_floats(g, c->sms);
+                    if (need > tc_floats) tc_floats = need;
+                    if (gemv_tc_tiles(g) > tc_tiles) tc_tiles = gemv_tc_tiles(g);
+                }
     }
     size_t sizes[] = {
         (size_t)f.max_ctx * (D / 2) * 4,                           // rope cos

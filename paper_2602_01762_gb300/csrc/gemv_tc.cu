@@ -433,8 +433,9 @@ __device__ __forceinline__ void chunk_to_lists(const float (&acc)[16], int row, 
 #pragma unroll 4
         for (int i = 0; i < kTileM / P; ++i) {
             const int r = i * P + q, u = tile * kTileM + r;
+            // a NaN logit is no candidate (as in the packed top-1 and the ring kernel)
             if (u < n_units) {
-                key_insert(l, pack_best(src[r], u));
+                if (src[r] == src[r]) key_insert(l, pack_best(src[r], u));
                 if (want_lse) lse_add(lm, ls, src[r]);
             }
         }

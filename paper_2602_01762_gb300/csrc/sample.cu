@@ -9,7 +9,7 @@
 // last CTA of the row merges them in CTA order and writes the token and
 // lse = log sum_i exp(z_i / T), so that p_draft(x) = exp(z_x / T - lse).
 //
-// Acceptance: one CTA per sequence walks the K drafted positions; x is
+// Acceptance: one cluster per sequence tests the K drafted positions; x is
 // accepted when r * p_draft(x) < p_target(x) (r < min(1, p_target /
 // p_draft)); the first rejected position draws its replacement from
 // max(0, p_target - p_draft) by an inverse-CDF search over the vocabulary (a
@@ -29,7 +29,6 @@ namespace prism {
 namespace {
 
 constexpr int kSampleThreads = 256;
-constexpr int kAcceptThreads = 1024;
 
 __device__ __forceinline__ uint64_t splitmix_at(uint64_t seed, uint64_t n) {
     uint64_t z = seed + (n + 1) * 0x9E3779B97F4A7C15ull;
@@ -140,112 +139,172 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
     }
 }
 
-// Inverse-CDF draw over w(0 .. V) (non-negative, not normalised), by the whole
-// CTA: thread t sums the contiguous chunk t, an inclusive scan gives the
-// chunk bounds, and the thread whose bounds hold u * total searches its
-// chunk.  Returns the token in every thread, or -1 when every weight is 0.
+// Inverse-CDF draw over the vocabulary by a cluster of kAccCtas CTAs.  The V
+// weights are cut into groups of 128 m consecutive tokens (m so that a CTA has
+// at most kAccGroups groups) and the groups into one contiguous range per CTA.
+// Each warp sums its groups with coalesced loads, several groups' loads in
+// flight; a scan of the CTA's group sums and the CTAs' totals, read through
+// distributed shared memory, gives every group its bounds on the cumulative
+// sum, and the one CTA whose range holds u * total searches the one group that
+// does, a warp at a time.  It is a chain of latencies on a few SMs: one CTA of
+// 1024 threads per sequence, each thread walking its own 126 tokens (128-byte
+// strides between neighbouring lanes, both rows through one SM), took
+// 64 us for 8 sequences of 128256 tokens; the cluster takes 13 us.
+constexpr int kAccCtas = 8;
+constexpr int kAccThreads = 512;
+constexpr int kAccWarps = kAccThreads / 32;
+constexpr int kAccGroups = 512;
+
+struct AccShared {
+    float gsum[kAccGroups];     // group sums, then their inclusive scan
+    float total;                // the CTA's sum
+    float wlast[kAccWarps];
+    float last;                 // last token of the CTA with a positive weight, -1: none (as a float's bits)
+    float tok;                  // the drawn token in the CTA that owns it, else -1 (as a float's bits)
+};
+
+// Returns the token in every thread of the cluster, or -1 when every weight is 0.
 template <typename W>
-__device__ int draw_block(W w, int V, float u, float *s_scan, int *s_tok) {
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int C = (V + kAcceptThreads - 1) / kAcceptThreads;
-    const int lo = min(V, tid * C), hi = min(V, lo + C);
-    float sum = 0.f;
+__device__ int draw_cluster(W w, int V, float u, AccShared &sh) {
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, r = blockIdx.x % kAccCtas;
+    int gs = 128;
+    while (((V + gs - 1) / gs + kAccCtas - 1) / kAccCtas > kAccGroups) gs *= 2;
+    const int ngroups = (V + gs - 1) / gs;
+    const int g0 = (int)((long)r * ngroups / kAccCtas), ng = (int)((long)(r + 1) * ngroups / kAccCtas) - g0;
     int last = -1;
-    for (int i = lo; i < hi; ++i) {
-        const float wi = w(i);
-        if (wi > 0.f) last = i;
-        sum += wi;
-    }
-    // inclusive scan: within the warp, then over the warp totals
-    float incl = sum;
+    for (int g = warp; g < ng; g += 2 * kAccWarps) {
+        float v[2][4] = {};
+        float sum[2] = {0.f, 0.f};
+        for (int o = 0; o < gs; o += 128) {
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const float x = __shfl_up_sync(0xFFFFFFFFu, incl, o);
-        if (lane >= o) incl += x;
+            for (int q = 0; q < 2; ++q)
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int gg = g + q * kAccWarps, i = (g0 + gg) * gs + o + 32 * j + lane;
+                    v[q][j] = gg < ng && i < V ? w(i) : 0.f;
+                    if (v[q][j] > 0.f) last = max(last, i);
+                }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) sum[q] += (v[q][0] + v[q][1]) + (v[q][2] + v[q][3]);
+        }
+#pragma unroll
+        for (int s = 16; s > 0; s >>= 1) {
+            sum[0] += __shfl_xor_sync(0xFFFFFFFFu, sum[0], s);
+            sum[1] += __shfl_xor_sync(0xFFFFFFFFu, sum[1], s);
+        }
+        if (lane == 0) {
+            sh.gsum[g] = sum[0];
+            if (g + kAccWarps < ng) sh.gsum[g + kAccWarps] = sum[1];
+        }
     }
-    if (lane == 31) s_scan[warp] = incl;
-    if (tid == 0) *s_tok = -1;
+    last = __reduce_max_sync(0xFFFFFFFFu, last);
+    if (lane == 0) sh.wlast[warp] = __int_as_float(last);
+    if (tid == 0) sh.tok = __int_as_float(-1);
     __syncthreads();
     if (warp == 0) {
-        float t = s_scan[lane];
+        float base = 0.f;
+        for (int g = 0; g < ng; g += 32) {
+            float c = g + lane < ng ? sh.gsum[g + lane] : 0.f;
 #pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const float x = __shfl_up_sync(0xFFFFFFFFu, t, o);
-            if (lane >= o) t += x;
+            for (int s = 1; s < 32; s <<= 1) {
+                const float x = __shfl_up_sync(0xFFFFFFFFu, c, s);
+                if (lane >= s) c += x;
+            }
+            if (g + lane < ng) sh.gsum[g + lane] = base + c;
+            base += __shfl_sync(0xFFFFFFFFu, c, 31);
         }
-        s_scan[lane] = t;
-    }
-    __syncthreads();
-    // chunk t covers [excl, incl); neighbours share each bound bit for bit
-    // (a warp's last bound is the warp-level sum the next warp starts from)
-    const float base = warp > 0 ? s_scan[warp - 1] : 0.f;
-    const float total = s_scan[kAcceptThreads / 32 - 1];
-    float excl = __shfl_up_sync(0xFFFFFFFFu, incl, 1);
-    if (lane == 0) excl = 0.f;
-    excl += base;
-    incl = lane == 31 ? s_scan[warp] : incl + base;
-    const float target = u * total;
-    if (total > 0.f && sum > 0.f && excl <= target && target < incl) {
-        float c = excl;
-        int tok = last;
-        for (int i = lo; i < hi; ++i) {
-            c += w(i);
-            if (c > target) { tok = i; break; }
+        const int l = __reduce_max_sync(0xFFFFFFFFu, lane < kAccWarps ? __float_as_int(sh.wlast[lane]) : -1);
+        if (lane == 0) {
+            sh.total = ng > 0 ? sh.gsum[ng - 1] : 0.f;
+            sh.last = __int_as_float(l);
         }
-        *s_tok = tok;
     }
-    __syncthreads();
-    int tok = *s_tok;
-    if (tok < 0 && total > 0.f) {
-        // u * total rounded onto the top of the range: the last positive weight
-        __syncthreads();
-        if (tid == 0) *s_tok = -1;
-        __syncthreads();
-        atomicMax(s_tok, last);
-        __syncthreads();
-        tok = *s_tok;
+    cluster_sync_all();
+    // CTA q covers [pre(q), pre(q) + total(q)), summed alike in every CTA
+    float total = 0.f, pre = 0.f;
+    int all_last = -1;
+#pragma unroll
+    for (int q = 0; q < kAccCtas; ++q) {
+        if (q == r) pre = total;
+        total += dsmem_ld(&sh.total, (uint32_t)q);
+        all_last = max(all_last, __float_as_int(dsmem_ld(&sh.last, (uint32_t)q)));
     }
-    __syncthreads();
+    const float target = u * total, own = sh.total;
+    if (warp == 0 && own > 0.f && pre <= target && target < pre + own) {
+        // the first group whose end lies beyond the target (the last one's does)
+        int g = 0;
+        for (; g < ng; g += 32) {
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, g + lane < ng && pre + sh.gsum[g + lane] > target);
+            if (m) { g += __ffs(m) - 1; break; }
+        }
+        g = min(g, ng - 1);
+        float c = g > 0 ? pre + sh.gsum[g - 1] : pre;
+        int tok = -1, seen = -1;
+        for (int o = 0; o < gs && tok < 0; o += 32) {
+            const int i = (g0 + g) * gs + o + lane;
+            const float wi = i < V ? w(i) : 0.f;
+            float in = wi;
+#pragma unroll
+            for (int s = 1; s < 32; s <<= 1) {
+                const float x = __shfl_up_sync(0xFFFFFFFFu, in, s);
+                if (lane >= s) in += x;
+            }
+            const unsigned m = __ballot_sync(0xFFFFFFFFu, wi > 0.f && c + in > target);
+            const unsigned pos = __ballot_sync(0xFFFFFFFFu, wi > 0.f);
+            if (m) tok = (g0 + g) * gs + o + __ffs(m) - 1;
+            if (pos) seen = (g0 + g) * gs + o + 31 - __clz(pos);
+            c += __shfl_sync(0xFFFFFFFFu, in, 31);
+        }
+        // the bounds came from sums in another order: the group's last positive weight
+        if (lane == 0) sh.tok = __int_as_float(tok >= 0 ? tok : seen);
+    }
+    cluster_sync_all();
+    int tok = -1;
+#pragma unroll
+    for (int q = 0; q < kAccCtas; ++q) tok = max(tok, __float_as_int(dsmem_ld(&sh.tok, (uint32_t)q)));
+    // u * total rounded onto the top of the range: the last positive weight
+    if (tok < 0 && total > 0.f) tok = all_last;
+    cluster_sync_all();         // every CTA has read before a second draw (or an exit) ends the values' life
     return tok;
 }
 
-__global__ void __launch_bounds__(kAcceptThreads) accept_sampled_kernel(const AcceptSampledArgs a) {
-    __shared__ float s_scan[kAcceptThreads / 32];
-    __shared__ int s_tok, s_dec;
-    const int b = blockIdx.x, tid = threadIdx.x, K = a.K, V = a.V;
+// One cluster per sequence.  Every CTA makes the K acceptance tests at once
+// (one lane each; K <= 16) and so finds the same first rejection.
+__global__ void __launch_bounds__(kAccThreads) accept_sampled_kernel(const AcceptSampledArgs a) {
+    __shared__ AccShared sh;
+    __shared__ int s_acc;
+    const int b = blockIdx.x / kAccCtas, rank = blockIdx.x % kAccCtas, tid = threadIdx.x, K = a.K, V = a.V;
     const uint64_t seed = *a.seed;
     const float inv_t = 1.0f / a.temperature;
-    int acc = 0, extra = -1;
-    for (; acc < K; ++acc) {
+    if (tid < 32) {
+        bool reject = false, bad = false;
+        if (tid < K) {
+            const size_t row = (size_t)b * K + tid;
+            int x = a.draft[row];
+            bad = x < 0 || x >= V;
+            if (bad) x = 0;
+            const float pd = expf(a.logits[row * V + x] * inv_t - a.lse[row]);
+            const float r = uniform01(seed, 2, (uint32_t)b, (uint32_t)tid, 0);
+            reject = !(r * pd < a.target[((size_t)b * (K + 1) + tid) * V + x]);
+        }
+        const unsigned rej = __ballot_sync(0xFFFFFFFFu, reject);
+        const int acc = rej ? __ffs(rej) - 1 : K;
+        if (bad && tid <= acc && rank == 0) set_err(a.err, kErrToken);   // positions the walk reaches
+        if (tid == 0) s_acc = acc;
+    }
+    __syncthreads();
+    const int acc = s_acc;
+    const float *pt = a.target + ((size_t)b * (K + 1) + acc) * V;
+    const float u = uniform01(seed, 3, (uint32_t)b, (uint32_t)acc, 0);
+    int extra = -1;
+    if (acc < K) {
         const size_t row = (size_t)b * K + acc;
         const float *z = a.logits + row * V;
-        const float *pt = a.target + ((size_t)b * (K + 1) + acc) * V;
         const float lse = a.lse[row];
-        if (tid == 0) {
-            int x = a.draft[row];
-            if (x < 0 || x >= V) {
-                set_err(a.err, kErrToken);
-                x = 0;
-            }
-            const float pd = expf(z[x] * inv_t - lse);
-            const float r = uniform01(seed, 2, (uint32_t)b, (uint32_t)acc, 0);
-            s_dec = r * pd < pt[x];
-        }
-        __syncthreads();
-        const bool accepted = s_dec;
-        __syncthreads();
-        if (accepted) continue;
-        const float u = uniform01(seed, 3, (uint32_t)b, (uint32_t)acc, 0);
-        extra = draw_block([&](int i) { return fmaxf(0.f, pt[i] - expf(z[i] * inv_t - lse)); }, V, u, s_scan, &s_tok);
-        if (extra < 0) extra = draw_block([&](int i) { return pt[i]; }, V, u, s_scan, &s_tok);
-        break;
+        extra = draw_cluster([&](int i) { return fmaxf(0.f, pt[i] - expf(z[i] * inv_t - lse)); }, V, u, sh);
     }
-    if (acc == K) {
-        const float *pt = a.target + ((size_t)b * (K + 1) + K) * V;
-        extra = draw_block([&](int i) { return pt[i]; }, V, uniform01(seed, 3, (uint32_t)b, (uint32_t)K, 0), s_scan,
-                           &s_tok);
-    }
-    if (tid == 0) {
+    if (extra < 0) extra = draw_cluster([&](int i) { return pt[i]; }, V, u, sh);
+    if (rank == 0 && tid == 0) {
         a.accept_len[b] = acc;
         for (int j = 0; j <= K; ++j) {
             int v = -1;
@@ -274,7 +333,18 @@ cudaError_t launch_sample(const SampleArgs &args, int B, cudaStream_t s, bool pd
 }
 
 cudaError_t launch_accept_sampled(const AcceptSampledArgs &a, cudaStream_t s) {
-    return launch_k(accept_sampled_kernel, dim3(a.B), dim3(kAcceptThreads), 0, s, false, a);
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(kAccCtas * a.B);
+    cfg.blockDim = dim3(kAccThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kAccCtas;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, accept_sampled_kernel, a);
 }
 
 }  // namespace prism

@@ -366,8 +366,8 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * weights instead of staging them whole in shared memory, its split-K sums
  * added by a separate finish kernel that also writes the next projection's
  * rows; at most 16 rows can be staged, and a staged projection's last CTA
- * per tile adds the sums itself; an LM head other than that streamed top-1
- * below (lm_stream) streams from max(this, 8) rows outside tree rounds), "attn_ctas_per_sm" (1..64, default 2: the fused attention
+ * per tile adds the sums itself; a greedy LM head other than that streamed
+ * top-1 below (lm_stream) streams from max(this, 8) rows outside tree rounds), "attn_ctas_per_sm" (1..64, default 2: the fused attention
  * kernel's cluster size halves while batch x KV heads x cluster size exceeds
  * this many CTAs per SM), "gemv_cuda_core" (for projections
  * not on the tcgen05 kernel: 1, the default, the CUDA-core TMA-ring kernel;
@@ -401,8 +401,8 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * "lm_stream" (1, the default: the top-1 LM head of a greedy round with up
  * to 16 rows streams them through its ring beside the weights, leaving the
  * ring the shared memory staged rows would take, and joins the rows' best
- * through the packed top-1 in the kernel; 0: as the LM head of a sampled
- * round, it stages fewer than max(tc_stream_rows, 8) rows (a top-1 then
+ * through the packed top-1 in the kernel; 0: it stages fewer than
+ * max(tc_stream_rows, 8) rows (a top-1 then
  * joins through the packed maximum) and streams more, selecting through
  * per-CTA lists and a merge kernel),
  * "tree_defer_merge" (1, the default: in tree rounds the LM head leaves its
@@ -438,7 +438,7 @@ prism_status prism_round_launches(prism_ctx *ctx, int32_t *n_launches);
  * max_kernels); *n_kernels receives the count; kernel_kind[i] (may be NULL)
  * receives a code: 0 fusion, 1 qkv, 2 rope/append, 3 attention (with the
  * fused option: RoPE, append and attention; no code-2 kernel then), 4 o-proj,
- * 5 gate/up, 6 down, 7 LM head + selection, 8 sampled draw (sampled rounds
+ * 5 gate/up, 6 down, 7 LM head + selection, 8 sampled draw after an LM head that does not draw itself (sampled rounds
  * only; this call profiles the greedy round).  Synchronises the stream. */
 prism_status prism_profile_round(prism_ctx *ctx, int32_t batch, const int32_t *tokens,
                                  const void *hidden, const int32_t *n_new, const int32_t *kv_len,

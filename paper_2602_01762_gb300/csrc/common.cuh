@@ -199,6 +199,20 @@ __device__ __forceinline__ void unpack_best(unsigned long long key, float &v, in
     id = (int)(0xFFFFFFFFu - (uint32_t)key);
 }
 
+// Random numbers of sampled rounds: output n of SplitMix64 from state `seed`,
+// and the uniform of (stream, b, k, i) in (0, 1) (prism.h).
+__device__ __forceinline__ uint64_t splitmix_at(uint64_t seed, uint64_t n) {
+    uint64_t z = seed + (n + 1) * 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
+__device__ __forceinline__ float uniform01(uint64_t seed, uint32_t stream, uint32_t b, uint32_t k, uint32_t i) {
+    const uint64_t n = ((uint64_t)stream << 60) | ((uint64_t)b << 40) | ((uint64_t)k << 32) | (uint64_t)i;
+    return ((float)(splitmix_at(seed, n) >> 41) + 0.5f) * (1.0f / 8388608.0f);
+}
+
 using Key = unsigned long long;
 
 __device__ __forceinline__ void key_clear(Key (&l)[kTopK]) {
@@ -332,6 +346,13 @@ struct GemvArgs {
     // 1: top-k lists are only published per CTA ([T][grid][8] in lm_part /
     // lm_part_id); the kernel that reads the selection merges them
     int defer_merge;
+    // a sampled round's LM head on the streamed kernel draws in its epilogue:
+    // seed word, 1 / T, per row and CTA (max, sum exp, best perturbed score, its
+    // id) [T][CTAs][4], and the draws' log-sum-exp [T][K] out; smp_part null: no draw
+    const uint64_t *smp_seed;
+    float smp_inv_t;
+    float *smp_part;
+    float *smp_lse;
     // 1: a streamed top-1 selection of up to 16 rows joins through the packed
     // atomic maximum in the kernel itself (no list merge kernel)
     int stream_top1;

@@ -418,11 +418,17 @@ constexpr int kTrMax = kTileM + 8;   // floats per transposed row, largest P
 // the 32 lanes of a scanning warp read 32 distinct banks.
 // With P = 8 every epilogue thread scans: thread e takes row c0 + e / 8.
 // With want_lse the scanning thread also adds each logit to its running
-// log-sum-exp (lm, ls) of that row.
-template <int P>
+// log-sum-exp (lm, ls) of that row.  SMP: of logit / T, and it keeps its best
+// Gumbel-perturbed logit / T (bv, bi; row b's stream at this step).
+struct Draw {
+    uint64_t seed;
+    float inv_t;
+    int step, row0;
+};
+template <int P, bool SMP>
 __device__ __forceinline__ void chunk_to_lists(const float (&acc)[16], int row, float *tr, int tile, int c0, int T,
                                                int n_units, bool dead, Key (&l)[kTopK], bool want_lse, float &lm,
-                                               float &ls) {
+                                               float &ls, const Draw &dr, float &bv, int &bi) {
     constexpr int S = kTileM + P;
 #pragma unroll
     for (int j = 0; j < 16; ++j) tr[j * S + row] = acc[j];
@@ -436,7 +442,15 @@ __device__ __forceinline__ void chunk_to_lists(const float (&acc)[16], int row, 
             // a NaN logit is no candidate (as in the packed top-1 and the ring kernel)
             if (u < n_units) {
                 if (src[r] == src[r]) key_insert(l, pack_best(src[r], u));
-                if (want_lse) lse_add(lm, ls, src[r]);
+                if constexpr (SMP) {
+                    const float v = src[r] * dr.inv_t;
+                    lse_combine(lm, ls, v, 1.f);
+                    const float p = v - logf(-logf(uniform01(dr.seed, 1, (uint32_t)(dr.row0 + t), (uint32_t)(dr.step - 1),
+                                                             (uint32_t)u)));
+                    if (better(p, u, bv, bi)) { bv = p; bi = u; }
+                } else if (want_lse) {
+                    lse_add(lm, ls, src[r]);
+                }
             }
         }
     }
@@ -458,6 +472,22 @@ __device__ __forceinline__ void lse_publish(const GemvArgs &a, float m, float s,
         pp[0] = m;
         pp[1] = s;
     }
+}
+
+// The same of a draw: (max, sum exp) and the best perturbed score with its id.
+__device__ __forceinline__ void draw_publish(const GemvArgs &a, float m, float s, float bv, int bi, int T, int t0,
+                                             int row0, int slot, int slots) {
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) {
+        const float m2 = __shfl_xor_sync(0xFFFFFFFFu, m, o), s2 = __shfl_xor_sync(0xFFFFFFFFu, s, o);
+        const float v2 = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
+        const int i2 = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
+        lse_combine(m, s, m2, s2);
+        if (better(v2, i2, bv, bi)) { bv = v2; bi = i2; }
+    }
+    const int e = threadIdx.x - 64, t = t0 + e / 8;
+    if ((e & 7) == 0 && t < T)
+        *(float4 *)(a.smp_part + ((size_t)(row0 + t) * slots + slot) * 4) = make_float4(m, s, bv, __int_as_float(bi));
 }
 
 // The CTA's list of each row: the P threads of a row merge theirs and write
@@ -518,14 +548,14 @@ __device__ __forceinline__ void gather_keys(const GemvArgs &a, int t, int grid, 
 
 // Row t's final top-k from a list every lane of the warp holds: lane r < topk
 // writes rank r.
-__device__ __forceinline__ void write_row(const GemvArgs &a, int t, const Key (&l)[kTopK]) {
+__device__ __forceinline__ void write_row(const GemvArgs &a, int t, const Key (&l)[kTopK], bool draft = true) {
     const int lane = threadIdx.x & 31;
     if (lane < a.topk) {
         float v;
         int id;
         unpack_best(key_at(l, lane), v, id);
         const size_t o = (size_t)t * a.K + a.step - 1;
-        if (lane == 0) a.draft_out[o] = id;
+        if (lane == 0 && draft) a.draft_out[o] = id;
         if (a.topk_ids) a.topk_ids[o * a.topk + lane] = id;
         if (a.topk_logits) a.topk_logits[o * a.topk + lane] = v;
     }
@@ -799,8 +829,10 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                     if constexpr (top1) {
                         top1_scan<NB>(acc[0], T, valid, u, thr_v, thr_i, s_val[ew], s_id[ew]);
                     } else {
-                        chunk_to_lists<8>(acc[0], row, &s_tr[0][0], tile, 0, T, a.n_units, dead, lst,
-                                          a.lse_part != nullptr, lse_m, lse_s);
+                        float bv = 0.f;
+                        int bi = 0;
+                        chunk_to_lists<8, false>(acc[0], row, &s_tr[0][0], tile, 0, T, a.n_units, dead, lst,
+                                                 a.lse_part != nullptr, lse_m, lse_s, Draw{}, bv, bi);
                     }
                 } else if (p.splits == 1) {
                     if (valid) {
@@ -888,7 +920,8 @@ __global__ void __launch_bounds__(kTcThreads, 1)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[kTcMaxStages], empty[kTcMaxStages], acc_full[2], acc_empty[2], mma_done;
     __shared__ uint32_t s_tmem;
-    constexpr bool TOPK = TK != 0, LISTS = TK == 2;   // TK: 0 none, 1 packed top-1, 2 top-k lists
+    // TK: 0 none, 1 packed top-1, 2 top-k lists, 3 top-k lists and the draw of a sampled round
+    constexpr bool TOPK = TK != 0, LISTS = TK >= 2, SMP = TK == 3;
     __shared__ float s_tr[LISTS ? 16 : 1][LISTS ? kTrMax : 1];
     __shared__ float s_val[TK == 1 ? 4 : 1][TK == 1 ? NB : 1];   // top-1: each epilogue warp's best per row
     __shared__ int s_id[TK == 1 ? 4 : 1][TK == 1 ? NB : 1];
@@ -1073,7 +1106,15 @@ __global__ void __launch_bounds__(kTcThreads, 1)
             // threads, 8 per row (each thread keeps one list per chunk position)
             constexpr int kNL = LISTS ? NB / 16 : 1;
             Key lst[kNL][kTopK];
-            float lse_m[kNL], lse_s[kNL];         // per chunk position, with a.lse_part
+            float lse_m[kNL], lse_s[kNL];         // per chunk position, with a.lse_part (or a draw)
+            float smp_v[SMP ? kNL : 1];           // a draw's best perturbed score per chunk position
+            int smp_i[SMP ? kNL : 1];
+            Draw draw{};
+            if constexpr (SMP) {
+                draw = Draw{*a.smp_seed, a.smp_inv_t, a.step, row0};
+#pragma unroll
+                for (int cc = 0; cc < kNL; ++cc) { smp_v[cc] = -INFINITY; smp_i[cc] = 0x7FFFFFFF; }
+            }
             if constexpr (LISTS) {
 #pragma unroll
                 for (int cc = 0; cc < kNL; ++cc) {
@@ -1125,8 +1166,9 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                                 if (c0 + tt < T) a.logits[((size_t)(row0 + c0 + tt) * a.K + a.step - 1) * a.vocab + u] = acc[tt];
                         }
                         if constexpr (LISTS)
-                            chunk_to_lists<8>(acc, row, &s_tr[0][0], tile, c0, T, a.n_units, dead, lst[cc],
-                                              a.lse_part != nullptr, lse_m[cc], lse_s[cc]);
+                            chunk_to_lists<8, SMP>(acc, row, &s_tr[0][0], tile, c0, T, a.n_units, dead, lst[cc],
+                                                   a.lse_part != nullptr, lse_m[cc], lse_s[cc], draw,
+                                                   smp_v[SMP ? cc : 0], smp_i[SMP ? cc : 0]);
                         else
                             top1_scan<kN1>(acc, T, valid, u, thr_v, thr_i, s_val[ew], s_id[ew]);
                     }
@@ -1170,8 +1212,12 @@ __global__ void __launch_bounds__(kTcThreads, 1)
                 // this CTA's list of every row; the cross-CTA merge is a separate kernel
 #pragma unroll
                 for (int cc = 0; cc < kNL; ++cc) {
-                    lists_publish<8>(a, lst[cc], T, 16 * cc, row0, RT ? item0 / p.n_rt : item0, RT ? step / p.n_rt : step);
-                    if (a.lse_part) lse_publish(a, lse_m[cc], lse_s[cc], T, 16 * cc, row0, RT ? item0 / p.n_rt : item0, RT ? step / p.n_rt : step);
+                    const int slot = RT ? item0 / p.n_rt : item0, slots = RT ? step / p.n_rt : step;
+                    lists_publish<8>(a, lst[cc], T, 16 * cc, row0, slot, slots);
+                    if constexpr (SMP)
+                        draw_publish(a, lse_m[cc], lse_s[cc], smp_v[cc], smp_i[cc], T, 16 * cc, row0, slot, slots);
+                    else if (a.lse_part)
+                        lse_publish(a, lse_m[cc], lse_s[cc], T, 16 * cc, row0, slot, slots);
                 }
             } else if constexpr (TK == 1) {
                 top1_join<kN1>(a, T, s_val, s_id, s_last);
@@ -1249,6 +1295,15 @@ __global__ void __launch_bounds__(128) topk_merge_kernel(const GemvArgs a, int g
         cv[b] = cc < ncand ? __ldcg(pv + cc) : 0.f;
         ci[b] = cc < ncand ? __ldcg(pi + cc) : -1;
     }
+    // a sampled round: warp 1 also merges the row's draw (lane l the partials l, l + 32, ...)
+    const bool smp = a.smp_part != nullptr;
+    constexpr int kS = 5;                           // partials per lane in the first batch (160 CTAs)
+    float4 sp[kS];
+    const float4 *spp = (const float4 *)a.smp_part + (size_t)t * grid;
+#pragma unroll
+    for (int b = 0; b < kS; ++b)
+        sp[b] = smp && w == 1 && lane + 32 * b < grid ? __ldcg(spp + lane + 32 * b)
+                                                      : make_float4(-INFINITY, 0.f, -INFINITY, __int_as_float(0x7FFFFFFF));
     uint4 *x = a.next_fuse ? (uint4 *)(a.next_x + (size_t)t * 2 * d) : nullptr;
     if (x) {
         // the h^ half of the next decode step's fusion row does not depend on the token
@@ -1291,12 +1346,42 @@ __global__ void __launch_bounds__(128) topk_merge_kernel(const GemvArgs a, int g
         // every lane ends with the merged list (write_row reads rank r from lane r)
 #pragma unroll 1
         for (int m = 1; m < 32; m <<= 1) key_merge_xor(l, m);
-        write_row(a, t, l);
-        if (lane == 0) {
+        write_row(a, t, l, !smp);
+        if (lane == 0 && !smp) {
             float v;
             int id;
             unpack_best(l[0], v, id);
             s_tok = id;
+        }
+    } else if (w == 1 && smp) {
+        float M = -INFINITY, S = 0.f, bv = -INFINITY;
+        int bi = 0x7FFFFFFF;
+        auto join = [&](float m2, float s2, float v2, int i2) {
+            lse_combine(M, S, m2, s2);
+            if (better(v2, i2, bv, bi)) { bv = v2; bi = i2; }
+        };
+#pragma unroll 1
+        for (int b = 0; b < kS; ++b) {
+            float4 q = sp[0];
+#pragma unroll
+            for (int c = 1; c < kS; ++c)
+                if (b == c) q = sp[c];
+            join(q.x, q.y, q.z, __float_as_int(q.w));
+        }
+#pragma unroll 1
+        for (int c = lane + 32 * kS; c < grid; c += 32) {
+            const float4 q = __ldcg(spp + c);
+            join(q.x, q.y, q.z, __float_as_int(q.w));
+        }
+#pragma unroll 1
+        for (int o = 16; o > 0; o >>= 1)
+            join(__shfl_xor_sync(0xFFFFFFFFu, M, o), __shfl_xor_sync(0xFFFFFFFFu, S, o),
+                 __shfl_xor_sync(0xFFFFFFFFu, bv, o), __shfl_xor_sync(0xFFFFFFFFu, bi, o));
+        if (lane == 0) {
+            const size_t o = (size_t)t * a.K + a.step - 1;
+            a.draft_out[o] = bi;
+            a.smp_lse[o] = M + logf(S);
+            s_tok = bi;
         }
     }
     if (x) {
@@ -1603,15 +1688,15 @@ void tcs_rows(int T, int RPW, bool topk, int &nb, int &n_rt) {
 }
 
 // The selection a streamed launch makes: 0 none, 1 the packed top-1 (one
-// 16-row tile of activation rows), 2 top-k lists.
+// 16-row tile of activation rows), 2 top-k lists, 3 lists and a sampled draw.
 int tcs_tk(const GemvArgs &a, int NB) {
     if (a.epi != kEpiTopK) return 0;
-    return a.stream_top1 && a.topk == 1 && a.best && NB == 16 ? 1 : 2;
+    return a.smp_part ? 3 : a.stream_top1 && a.topk == 1 && a.best && NB == 16 ? 1 : 2;
 }
 
 // static shared memory of a streamed kernel (barriers, top-1 bests, top-k lists)
 size_t tcs_static(int NB, int tk) {
-    return 512 + (tk == 2 ? (size_t)16 * kTrMax * 4 : tk == 1 ? (size_t)4 * NB * 8 : 64);
+    return 512 + (tk >= 2 ? (size_t)16 * kTrMax * 4 : tk == 1 ? (size_t)4 * NB * 8 : 64);
 }
 
 bool tcs_plan(const GemvArgs &a, int sms, TcPlan &p, int &grid, size_t &smem, int &NB) {
@@ -1687,7 +1772,9 @@ cudaError_t dispatch_tcs(const GemvArgs &a, const TcPlan &p, const CUtensorMap &
     // several row tiles: only the instances that tcs_rows gives them
     if (p.n_rt > 1) {
         if constexpr (NB == 64)
-            if (a.epi == kEpiTopK) return launch_k(gemv_tcs_kernel<NB, 1, 2, true>, g, b, smem, s, pdl, a, p, mw, mx);
+            if (a.epi == kEpiTopK)
+                return tcs_tk(a, NB) == 3 ? launch_k(gemv_tcs_kernel<NB, 1, 3, true>, g, b, smem, s, pdl, a, p, mw, mx)
+                                          : launch_k(gemv_tcs_kernel<NB, 1, 2, true>, g, b, smem, s, pdl, a, p, mw, mx);
         if constexpr (NB == 128)
             if (a.epi == kEpiSwiGLU) return launch_k(gemv_tcs_kernel<NB, 2, 0, true>, g, b, smem, s, pdl, a, p, mw, mx);
         if constexpr (NB == 192 || NB == 256)
@@ -1698,7 +1785,9 @@ cudaError_t dispatch_tcs(const GemvArgs &a, const TcPlan &p, const CUtensorMap &
     if (a.epi == kEpiTopK) {
         if constexpr (NB == 16)
             if (tcs_tk(a, NB) == 1) return launch_k(gemv_tcs_kernel<NB, 1, 1, false>, g, b, smem, s, pdl, a, p, mw, mx);
-        if constexpr (NB <= 64) return launch_k(gemv_tcs_kernel<NB, 1, 2, false>, g, b, smem, s, pdl, a, p, mw, mx);
+        if constexpr (NB <= 64)
+            return tcs_tk(a, NB) == 3 ? launch_k(gemv_tcs_kernel<NB, 1, 3, false>, g, b, smem, s, pdl, a, p, mw, mx)
+                                      : launch_k(gemv_tcs_kernel<NB, 1, 2, false>, g, b, smem, s, pdl, a, p, mw, mx);
         return cudaErrorInvalidValue;
     }
     if (a.epi == kEpiSwiGLU) {
@@ -1727,7 +1816,8 @@ cudaError_t prepare_gemv_tc_kernels() {
         e = set_tcs_attr<NB, RPW, TK, ##__VA_ARGS__>(                                                   \
             (int)std::min((size_t)b, (size_t)220 * 1024 - tcs_static(NB, TK)));
     PRISM_TCS(16, 1, 0) PRISM_TCS(32, 1, 0) PRISM_TCS(64, 1, 0) PRISM_TCS(128, 1, 0)
-    PRISM_TCS(192, 1, 0, true) PRISM_TCS(256, 1, 0, true) PRISM_TCS(128, 2, 0, true) PRISM_TCS(64, 1, 2, true)
+    PRISM_TCS(192, 1, 0, true) PRISM_TCS(256, 1, 0, true) PRISM_TCS(128, 2, 0, true) PRISM_TCS(64, 1, 2, true) PRISM_TCS(64, 1, 3, true)
+    PRISM_TCS(16, 1, 3) PRISM_TCS(32, 1, 3) PRISM_TCS(64, 1, 3)
     PRISM_TCS(256, 1, 0) PRISM_TCS(16, 2, 0) PRISM_TCS(32, 2, 0) PRISM_TCS(64, 2, 0)
     PRISM_TCS(128, 2, 0) PRISM_TCS(16, 1, 2) PRISM_TCS(32, 1, 2) PRISM_TCS(64, 1, 2)
 #undef PRISM_TCS
@@ -1837,7 +1927,7 @@ cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, f
         case 192: e = dispatch_tcs<192>(a, p, mw, mx, grid, smem, s, pdl); break;
         default: e = dispatch_tcs<256>(a, p, mw, mx, grid, smem, s, pdl); break;
     }
-    if (e == cudaSuccess && a.epi == kEpiTopK && tcs_tk(a, NB) == 2) {
+    if (e == cudaSuccess && a.epi == kEpiTopK && tcs_tk(a, NB) >= 2) {
         GemvArgs m = a;
         m.next_fuse = a.next_fuse && a.next_x && a.d % 8 == 0;
         if (!a.defer_merge) e = launch_k(topk_merge_kernel, dim3(a.T), dim3(128), 0, s, true, m, grid / p.n_rt);

@@ -109,7 +109,7 @@ struct prism_ctx {
     int *lm_id = nullptr;
     int *counters = nullptr;  // [max_batch * Hkv] attention + [1] LM head
     unsigned long long *lm_best = nullptr;  // [max_batch] LM head top-1 keys (left at zero)
-    float *sample_part = nullptr;           // [max_batch, kSampleMaxBlocks, 4] sampled-draft partials
+    float *sample_part = nullptr;           // [max_batch, max(LM-head CTAs, kSampleMaxBlocks), 4] sampled-draft partials
     int *sample_ctr = nullptr;              // [max_batch] sampled-draft tickets (left at zero)
     // tree drafting (max_tree_width > 0): w rows per sequence, frontier and candidate pool
     int tree_rows = 0;                      // max_batch * max(1, max_tree_width)
@@ -266,13 +266,15 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
         // the top-1 LM head streams its rows from one row on with lm_stream
         // (not in sampled rounds, whose draw reads the logits it writes)
         const bool lm1 = c->lm_stream && g.stream_top1 && g.epi == kEpiTopK && g.topk == 1 && g.best;
-        // any other LM head outside tree rounds (sampled rounds; greedy ones with
-        // lm_stream off) keeps fewer than 8 rows staged:
-        // at batch 1 a sampled round took 1371 us with every row streamed against
-        // 1360 us with every row staged, while streaming the other projections
-        // alone saves 17 us in a greedy round
-        const int rows_min = g.epi == kEpiTopK && !lm1 && !(r.tree_w > 0) ? std::max(c->tc_stream_rows, 8)
-                                                                            : c->tc_stream_rows;
+        // any other greedy LM head (top-k lists; lm_stream off) keeps fewer than
+        // 8 rows staged, where its lists merge without another kernel; a sampled
+        // one streams, and draws in its epilogue and merge kernel (Llama-3-8B
+        // shape, round and acceptance at batch 1 / 4 / 8 / 16, with the sampling
+        // kernel reading the logits back: 1427 / 1587 / 1563 / 1642 us; drawing in
+        // the LM head: 1347 / 1477 / 1469 / 1511 us, of which the acceptance's own
+        // change is 50)
+        const int rows_min = g.epi == kEpiTopK && !lm1 && !g.smp_part && !(r.tree_w > 0)
+                                 ? std::max(c->tc_stream_rows, 8) : c->tc_stream_rows;
         if (!(tm && want_tc(g) && c->tc_ready && c->bf16 && (g.T >= rows_min || lm1) &&
               gemv_tcs_supported(g, c->sms)))
             return false;
@@ -489,6 +491,15 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
         g.draft_out = r.draft;
         g.topk_ids = r.topk_ids;
         g.topk_logits = r.topk_logits;
+        if (r.temperature > 0.f) {
+            // the streamed kernel draws x^_k itself; after any other LM head the
+            // sampling kernel does
+            g.smp_seed = r.seed;
+            g.smp_inv_t = 1.0f / r.temperature;
+            g.smp_part = c->sample_part;
+            g.smp_lse = r.lse;
+            if (!on_tcs(g, c->tm_lm_ok ? &c->tm_lm : nullptr)) g.smp_part = nullptr;
+        }
         if (tree) {
             // rows b * w + j of [B * w, .] buffers: at step 1 (one row per
             // sequence) K = w puts row b at b * w; later steps index by row
@@ -676,7 +687,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
                  lm_tm);
         after(6);
         if (e != cudaSuccess) break;
-        const bool chain_next = k < K && !tree && !(r.temperature > 0.f);
+        const bool chain_next = k < K && !tree && (!(r.temperature > 0.f) || gl.smp_part);
         const GemvArgs gn = chain_next ? fusion_args(k + 1) : GemvArgs{};
         e = proj(with_pf(gl, pf(k < K ? c->steps[k].w_fuse : nullptr, (size_t)d * 2 * d)), lm_tm, c->lm_grid, pdl,
                  chain_next ? &gn : nullptr, chain_next ? step_tm(k + 1, 0) : nullptr);
@@ -699,7 +710,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             continue;
         }
 
-        if (r.temperature > 0.f) {
+        if (r.temperature > 0.f && !gl.smp_part) {
             // x^_k drawn from softmax(z / T): replaces the argmax before the next step reads it
             SampleArgs sa{};
             sa.logits = r.logits;
@@ -825,7 +836,7 @@ prism_status prism_create(const prism_config *cfg, int32_t device, prism_ctx **o
         tc_floats * 4,                                             // tensor-core split-K partials
         (size_t)tc_tiles * 4,                                      // tensor-core tile tickets
         T1 * 2 * d * es,                                           // streamed-kernel activation rows
-        B * (size_t)kSampleMaxBlocks * 4 * 4,                      // sampled-draft partials
+        B * (size_t)std::max(c->lm_grid, kSampleMaxBlocks) * 4 * 4,  // sampled-draft partials
         B * 4,                                                     // sampled-draft tickets
         tree_on * Bw * 2 * d * es,                                 // tree fusion inputs
         tree_on * Bw * f.vocab * 4,                                // tree row logits

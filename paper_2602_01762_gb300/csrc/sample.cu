@@ -1,13 +1,14 @@
 // Sampled drafting and speculative-sampling acceptance (Sec. 2 at a
 // temperature T > 0), sm_103a.
 //
-// Drafting: after the LM head of step k has written its logits z, each draft
-// token is drawn from p_draft = softmax(z / T) by the Gumbel-max rule: the
+// Drafting: each draft token is drawn from p_draft = softmax(z / T) by the Gumbel-max rule: the
 // argmax of z_i / T + G_i with G_i = -log(-log U_i) is distributed as
 // softmax(z / T).  The logits of one row are split over many CTAs; each keeps
 // a running (max, sum of exp) of z / T and its best perturbed score, and the
 // last CTA of the row merges them in CTA order and writes the token and
-// lse = log sum_i exp(z_i / T), so that p_draft(x) = exp(z_x / T - lse).
+// lse = log sum_i exp(z_i / T), so that p_draft(x) = exp(z_x / T - lse).  A
+// streamed tcgen05 LM head draws in its own epilogue (gemv_tc.cu); sample_kernel
+// here reads the logits back after any other LM head.
 //
 // Acceptance: one cluster per sequence tests the K drafted positions; x is
 // accepted when r * p_draft(x) < p_target(x) (r < min(1, p_target /
@@ -30,18 +31,6 @@ namespace {
 
 constexpr int kSampleThreads = 256;
 
-__device__ __forceinline__ uint64_t splitmix_at(uint64_t seed, uint64_t n) {
-    uint64_t z = seed + (n + 1) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-__device__ __forceinline__ float uniform01(uint64_t seed, uint32_t stream, uint32_t b, uint32_t k, uint32_t i) {
-    const uint64_t n = ((uint64_t)stream << 60) | ((uint64_t)b << 40) | ((uint64_t)k << 32) | (uint64_t)i;
-    return ((float)(splitmix_at(seed, n) >> 41) + 0.5f) * (1.0f / 8388608.0f);
-}
-
 // (max, sum of exp(v - max)) of two parts, combined.
 __device__ __forceinline__ void lse_merge(float &m, float &s, float m2, float s2) {
     if (m2 == -INFINITY) return;
@@ -49,8 +38,6 @@ __device__ __forceinline__ void lse_merge(float &m, float &s, float m2, float s2
     if (m2 > m) { s = s * expf(m - m2) + s2; m = m2; }
     else s += s2 * expf(m2 - m);
 }
-// better perturbed score: larger, ties to the lower id
-__device__ __forceinline__ bool score_better(float v, int i, float bv, int bi) { return v > bv || (v == bv && i < bi); }
 
 // grid (blocks per row, B); a CTA takes `chunk` consecutive logits of row b.
 __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs a) {
@@ -72,7 +59,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
         lse_merge(m, s, v, 1.f);
         const float u = uniform01(seed, 1, (uint32_t)b, (uint32_t)(a.step - 1), (uint32_t)i);
         const float g = v - logf(-logf(u));
-        if (score_better(g, i, bv, bi)) { bv = g; bi = i; }
+        if (better(g, i, bv, bi)) { bv = g; bi = i; }
     }
     // block: warps in a fixed tree, then warp 0 over the warps in order
 #pragma unroll
@@ -81,14 +68,14 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
         const float v2 = __shfl_xor_sync(0xFFFFFFFFu, bv, o);
         const int i2 = __shfl_xor_sync(0xFFFFFFFFu, bi, o);
         lse_merge(m, s, m2, s2);
-        if (score_better(v2, i2, bv, bi)) { bv = v2; bi = i2; }
+        if (better(v2, i2, bv, bi)) { bv = v2; bi = i2; }
     }
     if (lane == 0) { s_m[warp] = m; s_s[warp] = s; s_v[warp] = bv; s_i[warp] = bi; }
     __syncthreads();
     if (tid == 0) {
         for (int w = 1; w < kSampleThreads / 32; ++w) {
             lse_merge(m, s, s_m[w], s_s[w]);
-            if (score_better(s_v[w], s_i[w], bv, bi)) { bv = s_v[w]; bi = s_i[w]; }
+            if (better(s_v[w], s_i[w], bv, bi)) { bv = s_v[w]; bi = s_i[w]; }
         }
         float *part = a.part + ((size_t)b * a.max_blocks + blk) * 4;
         part[0] = m;
@@ -121,7 +108,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
         lse_merge(M, S, pm[i], ps[i]);
-        if (score_better(pv[i], pi[i], BV, BI)) { BV = pv[i]; BI = pi[i]; }
+        if (better(pv[i], pi[i], BV, BI)) { BV = pv[i]; BI = pi[i]; }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
@@ -129,7 +116,7 @@ __global__ void __launch_bounds__(kSampleThreads) sample_kernel(const SampleArgs
         const float v2 = __shfl_xor_sync(0xFFFFFFFFu, BV, o);
         const int i2 = __shfl_xor_sync(0xFFFFFFFFu, BI, o);
         lse_merge(M, S, m2, s2);
-        if (score_better(v2, i2, BV, BI)) { BV = v2; BI = i2; }
+        if (better(v2, i2, BV, BI)) { BV = v2; BI = i2; }
     }
     if (lane == 0) {
         const size_t o = (size_t)b * a.K + a.step - 1;

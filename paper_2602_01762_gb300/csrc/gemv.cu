@@ -1,4 +1,5 @@
-// Weight-streaming projections of the PRISM draft step (sm_103a).
+// Weight-streaming projections of the PRISM draft step on the CUDA cores, bf16
+// (sm_103a); fp32 ones are in gemv_f32.cu.
 //
 // Every projection of a draft step (fusion F, QKV, O, gate/up, down, LM head;
 // Sec. 3.2 and the Llama block) is y[t] = W x[t] for a handful of activation
@@ -106,13 +107,6 @@ __device__ __forceinline__ void dot16B<uint16_t>(unsigned long long &a0, unsigne
     ffma2(a0, pack2(w.z << 16, w.z & 0xFFFF0000u), pack2(x.z << 16, x.z & 0xFFFF0000u));
     ffma2(a1, pack2(w.w << 16, w.w & 0xFFFF0000u), pack2(x.w << 16, x.w & 0xFFFF0000u));
 }
-template <>
-__device__ __forceinline__ void dot16B<float>(unsigned long long &a0, unsigned long long &a1, const uint4 &w,
-                                              const uint4 &x) {
-    ffma2(a0, pack2(w.x, w.y), pack2(x.x, x.y));
-    ffma2(a1, pack2(w.z, w.w), pack2(x.z, x.w));
-}
-
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
@@ -249,7 +243,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemv_kernel(const GemvArgs a, con
 
     constexpr int VEC = Elem<WT>::kPerVec;
     constexpr int U = TC <= 2 ? 4 : (TC == 4 ? 2 : 1);
-    static_assert(sizeof(WT) == 2 || sizeof(WT) == 4, "weight type");
+    static_assert(sizeof(WT) == 2, "weight type");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int R = plan.R, S = plan.stages;
     const size_t row_bytes = (size_t)a.kin * sizeof(WT);
@@ -593,7 +587,7 @@ bool make_plan(const GemvArgs &a, bool bf16, int &tc, RingPlan &pl, size_t &smem
 
 cudaError_t prepare_gemv_kernels() {
     cudaError_t e = set_smem_attrs<uint16_t>((int)kSmemAlone);
-    if (e == cudaSuccess) e = set_smem_attrs<float>((int)kSmemAlone);
+    if (e == cudaSuccess) e = prepare_gemv_f32_kernels();
     if (e == cudaSuccess) e = prepare_gemv_mma_kernels();
     return e;
 }
@@ -601,30 +595,28 @@ cudaError_t prepare_gemv_kernels() {
 bool gemv_supported(const GemvArgs &a, bool bf16) {
     // launch_gemv takes the mma.sync kernel only when the CUDA-core one is not forced
     if (bf16 && !a.force_cuda_core && gemv_mma_supported(a)) return true;
+    // the limit on the contraction's length is the ring's for fp32 too, which
+    // gemv_f32.cu then always meets
     int tc;
     RingPlan pl;
     size_t smem;
     return make_plan(a, bf16, tc, pl, smem);
 }
 
-// bf16 projections whose contraction length is a multiple of 32 run on the
-// tensor-core kernel (gemv_mma.cu); the rest on the CUDA-core ring kernel.
+// fp32 projections run in gemv_f32.cu, bf16 ones whose contraction length is a
+// multiple of 32 on the mma.sync kernel (gemv_mma.cu) unless the CUDA-core
+// kernel is forced; the rest on the CUDA-core ring kernel.
 cudaError_t launch_gemv(const GemvArgs &a, bool bf16, int grid, cudaStream_t s, bool pdl) {
+    if (!bf16) return launch_gemv_f32(a, grid, s, pdl);
     if (bf16 && !a.force_cuda_core && gemv_mma_supported(a)) return launch_gemv_mma(a, grid, s, pdl);
     int tc;
     RingPlan pl;
     size_t smem;
     if (!make_plan(a, bf16, tc, pl, smem)) return cudaErrorInvalidValue;
-    if (bf16) {
-        if (tc == 1) return dispatch_kind<uint16_t, 1>(a, pl, grid, smem, s, pdl);
-        if (tc == 2) return dispatch_kind<uint16_t, 2>(a, pl, grid, smem, s, pdl);
-        if (tc == 4) return dispatch_kind<uint16_t, 4>(a, pl, grid, smem, s, pdl);
-        return dispatch_kind<uint16_t, 8>(a, pl, grid, smem, s, pdl);
-    }
-    if (tc == 1) return dispatch_kind<float, 1>(a, pl, grid, smem, s, pdl);
-    if (tc == 2) return dispatch_kind<float, 2>(a, pl, grid, smem, s, pdl);
-    if (tc == 4) return dispatch_kind<float, 4>(a, pl, grid, smem, s, pdl);
-    return dispatch_kind<float, 8>(a, pl, grid, smem, s, pdl);
+    if (tc == 1) return dispatch_kind<uint16_t, 1>(a, pl, grid, smem, s, pdl);
+    if (tc == 2) return dispatch_kind<uint16_t, 2>(a, pl, grid, smem, s, pdl);
+    if (tc == 4) return dispatch_kind<uint16_t, 4>(a, pl, grid, smem, s, pdl);
+    return dispatch_kind<uint16_t, 8>(a, pl, grid, smem, s, pdl);
 }
 
 }  // namespace prism

@@ -1884,6 +1884,10 @@ size_t gemv_tcs_workspace_floats(const GemvArgs &a, int sms) {
     return (size_t)p.splits * (a.epi == kEpiSwiGLU ? 2 : 1) * a.T * a.n_units;
 }
 
+cudaError_t launch_topk_merge(const GemvArgs &a, int slots, cudaStream_t s) {
+    return launch_k(topk_merge_kernel, dim3(a.T), dim3(128), 0, s, true, a, slots);
+}
+
 cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, float *part, int *tile_ctr,
                             uint16_t *xbuf, cudaStream_t s, bool pdl, bool *next_done) {
     if (next_done) *next_done = false;
@@ -1930,7 +1934,7 @@ cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, f
     if (e == cudaSuccess && a.epi == kEpiTopK && tcs_tk(a, NB) >= 2) {
         GemvArgs m = a;
         m.next_fuse = a.next_fuse && a.next_x && a.d % 8 == 0;
-        if (!a.defer_merge) e = launch_k(topk_merge_kernel, dim3(a.T), dim3(128), 0, s, true, m, grid / p.n_rt);
+        if (!a.defer_merge) e = launch_topk_merge(m, grid / p.n_rt, s);
         if (e == cudaSuccess && next_done) *next_done = !a.defer_merge && m.next_fuse != 0;
     }
     if (e == cudaSuccess && p.defer) {

@@ -380,6 +380,46 @@ __device__ __forceinline__ void fa_load(const FusedAttnArgs &a, int b, int g, in
     }
 }
 
+// Four consecutive elements stored as the cache's type.
+__device__ __forceinline__ void store4(uint16_t *p, float x, float y, float z, float w) {
+    *(uint2 *)p = make_uint2(pack_bf16x2(x, y), pack_bf16x2(z, w));
+}
+__device__ __forceinline__ void store4(float *p, float x, float y, float z, float w) {
+    *(float4 *)p = make_float4(x, y, z, w);
+}
+
+// The new rows [first, first + n) of head (b, g), row row0 of qkv the first,
+// that lie in this CTA's keys [j0, j1): keys rotated, keys and values into the
+// cache.  The whole CTA takes them side by side, four rotary pairs and eight
+// values a thread, every load of a step issued before any is used: a step is
+// one round trip for blockDim / (D / 8) rows.  (Row after row, each a round
+// trip or two, a prompt of 1000 rows held the kernel for 168 us: the round 1622 us, 1495 now.)
+template <typename WT, int D>
+__device__ __forceinline__ void append_rows(const FusedAttnArgs &a, int b, int g, int row0, int first, int n, int j0,
+                                            int j1, bool report) {
+    constexpr int half = D / 2, Q = D / 8;
+    const int H = a.Hq + 2 * a.Hkv;
+    // positions outside the cache: no rank owns them
+    if (report && threadIdx.x == 0 && (first < 0 || (long)first + n > a.max_ctx)) set_err(a.err, kErrCache);
+    const int lo = max(first, j0), hi = (int)min((long)first + n, (long)j1);
+#pragma unroll 2
+    for (int e = threadIdx.x; e < (hi - lo) * Q; e += blockDim.x) {
+        const int pos = lo + e / Q, q = e % Q;
+        const float *xk = a.qkv + ((size_t)(row0 + pos - first) * H + a.Hq + g) * D, *xv = xk + (size_t)a.Hkv * D;
+        const float4 x0 = __ldcg((const float4 *)xk + q), x1 = __ldcg((const float4 *)(xk + half) + q);
+        const float4 v0 = __ldcg((const float4 *)xv + 2 * q), v1 = __ldcg((const float4 *)xv + 2 * q + 1);
+        const float4 c = __ldg((const float4 *)(a.rope_cos + (size_t)pos * half) + q);
+        const float4 s = __ldg((const float4 *)(a.rope_sin + (size_t)pos * half) + q);
+        const size_t o = (((size_t)b * a.Hkv + g) * a.max_ctx + pos) * D;
+        WT *kc = (WT *)a.k_cache + o, *vc = (WT *)a.v_cache + o;
+        store4(kc + 4 * q, x0.x * c.x - x1.x * s.x, x0.y * c.y - x1.y * s.y, x0.z * c.z - x1.z * s.z, x0.w * c.w - x1.w * s.w);
+        store4(kc + half + 4 * q, x1.x * c.x + x0.x * s.x, x1.y * c.y + x0.y * s.y, x1.z * c.z + x0.z * s.z,
+               x1.w * c.w + x0.w * s.w);
+        store4(vc + 8 * q, v0.x, v0.y, v0.z, v0.w);
+        store4(vc + 8 * q + 4, v1.x, v1.y, v1.z, v1.w);
+    }
+}
+
 // p4[i % 4] += q[i] * k[i] over one 16-byte vector of keys (q broadcast).
 template <typename WT>
 __device__ __forceinline__ void dot4(float (&p4)[4], const float *q, const uint4 &k);
@@ -451,27 +491,7 @@ __global__ void __launch_bounds__(kFusedThreads, 1) fused_attention_kernel(const
     pdl_wait();
 
     // append the new rows this rank owns: positions L .. L+n-1 (prefill) or qp
-    const int first_new = a.prefill ? L : qp, n_rows = a.prefill ? n : 1;
-    for (int i = 0; i < n_rows; ++i) {
-        const int pos = first_new + i;
-        if (pos < 0 || pos >= a.max_ctx) {              // no rank owns it: rank 0 reports
-            if (r == 0 && tid == 0) set_err(a.err, kErrCache);
-            continue;
-        }
-        if (pos < j0 || pos >= j1) continue;
-        const int row = a.prefill ? b * a.max_new + i : b;
-        const float *xk = a.qkv + (size_t)row * H * D + (size_t)(a.Hq + g) * D;
-        const float *xv = a.qkv + (size_t)row * H * D + (size_t)(a.Hq + a.Hkv + g) * D;
-        WT *kc = (WT *)a.k_cache + (((size_t)b * a.Hkv + g) * a.max_ctx + pos) * D;
-        WT *vc = (WT *)a.v_cache + (((size_t)b * a.Hkv + g) * a.max_ctx + pos) * D;
-        for (int j = tid; j < half; j += kFusedThreads) {
-            const float c = a.rope_cos[(size_t)pos * half + j], sn = a.rope_sin[(size_t)pos * half + j];
-            const float x0 = xk[j], x1 = xk[j + half];
-            Elem<WT>::store(kc, j, x0 * c - x1 * sn);
-            Elem<WT>::store(kc, j + half, x1 * c + x0 * sn);
-        }
-        for (int j = tid; j < D; j += kFusedThreads) Elem<WT>::store(vc, j, xv[j]);
-    }
+    append_rows<WT, D>(a, b, g, a.prefill ? b * a.max_new : b, a.prefill ? L : qp, a.prefill ? n : 1, j0, j1, r == 0);
     // rotated queries of the heads sharing g, at qp, scaled by 1/sqrt(D)
     {
         const int row = a.prefill ? b * a.max_new + n - 1 : b;
@@ -926,27 +946,7 @@ __global__ void __launch_bounds__(TaCfg<W>::kThreads, TaCfg<W>::kMinBlocks)
     pdl_wait();
 
     // append the new rows this rank owns
-    const int first_new = a.prefill ? L : qp, n_rows = a.prefill ? n : 1;
-    for (int i = 0; i < n_rows; ++i) {
-        const int pos = first_new + i;
-        if (pos < 0 || pos >= a.max_ctx) {
-            if (r == 0 && tid == 0) set_err(a.err, kErrCache);
-            continue;
-        }
-        if (pos < j0 || pos >= j1) continue;
-        const int row = a.prefill ? b * a.max_new + i : b;
-        const float *xk = a.qkv + (size_t)row * H * D + (size_t)(a.Hq + g) * D;
-        const float *xv = a.qkv + (size_t)row * H * D + (size_t)(a.Hq + a.Hkv + g) * D;
-        uint16_t *kc = (uint16_t *)a.k_cache + (((size_t)b * a.Hkv + g) * a.max_ctx + pos) * D;
-        uint16_t *vc = (uint16_t *)a.v_cache + (((size_t)b * a.Hkv + g) * a.max_ctx + pos) * D;
-        for (int j = tid; j < half; j += kTaThreads) {
-            const float c = a.rope_cos[(size_t)pos * half + j], sn = a.rope_sin[(size_t)pos * half + j];
-            const float x0 = xk[j], x1 = xk[j + half];
-            kc[j] = f32_to_bf16(x0 * c - x1 * sn);
-            kc[j + half] = f32_to_bf16(x1 * c + x0 * sn);
-        }
-        for (int j = tid; j < D; j += kTaThreads) vc[j] = f32_to_bf16(xv[j]);
-    }
+    append_rows<uint16_t, D>(a, b, g, a.prefill ? b * a.max_new : b, a.prefill ? L : qp, a.prefill ? n : 1, j0, j1, r == 0);
     // queries (heads >= G zero), rotated and scaled by 1/sqrt(D)
     {
         const int row = a.prefill ? b * a.max_new + n - 1 : b;

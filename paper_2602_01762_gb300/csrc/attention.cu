@@ -1107,6 +1107,358 @@ __global__ void __launch_bounds__(TaCfg<W>::kThreads, TaCfg<W>::kMinBlocks)
     cluster_sync_all();
 }
 
+// Tree attention for bf16 caches, at step k >= 2 of a tree round: the w rows of
+// a sequence (tree.cu) share its cache, so one cluster of CTAs per (sequence,
+// KV head) takes all NQ = w * G row-head pairs over one pass of the keys.  The
+// key loop is the chain kernel's above (TMA ring, keys in M, per-warp online
+// softmax, merge through distributed shared memory) with the pairs in N as NTN
+// n8 tiles (pairs past NQ are zero queries), the queries' hi and lo parts in
+// shared memory instead of registers, and a key at or past `base` visible to a
+// pair only where its row's ancestor mask says so.
+// The kernel this replaces gave 128 keys to a CTA, wrote every CTA's sums to
+// memory and had the last CTA of a (sequence, head) read them back: at 17
+// splits that tail was most of the launch (24 us at batch 1 and context 2048, 43
+// at 4 sequences, for 2 and 3 us of bytes).  Tree rounds of 4 branches: batch 1,
+// 6 steps, context 2048: 1705 us before, 1647 now; 4 sequences, 4 steps, context
+// 512 to 2048: 1226 and 1191.
+template <int D, int NTN>
+__global__ void __launch_bounds__(TaCfg<8>::kThreads, 1)
+    tree_attention_cluster_kernel(const TreeArgs a, const __grid_constant__ CUtensorMap tk,
+                                  const __grid_constant__ CUtensorMap tv) {
+    constexpr int W = 8, kC = TaCfg<W>::kC, kThr = TaCfg<W>::kThreads, NH = D / 64, NT = D / 16, NP = 8 * NTN;
+    constexpr uint32_t kBox = kC * 128, kStage = 2 * NH * kBox;
+    constexpr int QW = D / 2 + 4;                     // words per query row: conflict-free fragment reads
+    extern __shared__ __align__(1024) uint8_t smem_raw[];
+    __shared__ __align__(8) uint64_t full[kTaStages], empty[kTaStages];
+    __shared__ unsigned long long s_mask[NP];         // each pair's row mask
+    uint8_t *ring = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+    uint32_t *qh = (uint32_t *)(ring + kTaStages * kStage), *ql = qh + NP * QW;  // [NP][QW] bf16 pairs
+    float *po = (float *)qh;                          // [NP][D] this rank's output, after the key loop
+    float *pm = (float *)(ql + NP * QW), *pl = pm + NP;
+    float *wo = (float *)ring;                        // [warp][NP][D], after the key loop
+    float *wm = wo + W * NP * D, *wl = wm + W * NP;   // [warp][NP]
+
+    const int r = blockIdx.x, g = blockIdx.y, b = blockIdx.z, CS = gridDim.x;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int half = D / 2, H = a.Hq + 2 * a.Hkv, G = a.Hq / a.Hkv, NQ = a.w * G;
+    const long lim = wait_bound(a.wait_polls, kAttnWaitLimit);
+    pdl_trigger();
+    const int n = clamp_n(a.n_new, b, a.max_new, a.err), L = a.kv_len[b];
+    const int base = L + n, new0 = base + (a.step - 2) * a.w, pos = base + a.step - 2;
+    // keys [0, P); a negative length is reported and attends to nothing
+    const bool bad = L < 0 || (long)base + (long)(a.step - 1) * a.w > a.max_ctx;
+    const int P = L < 0 ? 0 : min(base + (a.step - 1) * a.w, a.max_ctx);
+    const int j0 = (int)((long)r * P / CS), j1 = (int)((long)(r + 1) * P / CS);
+    const int nst = (j1 - j0 + kC - 1) / kC;
+    const uint32_t ring_s = sa(ring);
+    auto load = [&](int i) {
+        const int s = i % kTaStages, j = j0 + i * kC, z = b * a.Hkv + g;
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(sa(&full[s])), "r"(kStage)
+                     : "memory");
+        const uint32_t kd = ring_s + (uint32_t)s * kStage, vd = kd + NH * kBox;
+#pragma unroll
+        for (int h = 0; h < NH; ++h)
+#pragma unroll
+            for (int q = 0; q < kC / kTaBoxRows; ++q) {
+                const uint32_t o = h * kBox + q * kTaBoxRows * 128;
+                asm volatile(
+                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+                    "%3, %4}], [%5];" ::"r"(kd + o), "l"((uint64_t)&tk), "r"(h * 64), "r"(j + q * kTaBoxRows), "r"(z),
+                    "r"(sa(&full[s]))
+                    : "memory");
+                asm volatile(
+                    "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+                    "%3, %4}], [%5];" ::"r"(vd + o), "l"((uint64_t)&tv), "r"(h * 64), "r"(j + q * kTaBoxRows), "r"(z),
+                    "r"(sa(&full[s]))
+                    : "memory");
+            }
+    };
+    const bool producer = tid == W * 32;
+    if (producer) {
+        for (int s = 0; s < kTaStages; ++s) {
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sa(&full[s])));
+            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(sa(&empty[s])), "r"(W));
+        }
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tk) : "memory");
+        asm volatile("prefetch.tensormap [%0];" ::"l"((uint64_t)&tv) : "memory");
+    }
+    __syncthreads();
+    // stages made only of rows committed before the round do not wait
+    int pre = 0;
+    while (pre < kTaStages && pre < nst && min(j0 + (pre + 1) * kC, j1) <= L) ++pre;
+    if (producer)
+        for (int i = 0; i < pre; ++i) load(i);
+    pdl_wait();
+
+    if (bad && r == 0 && g == 0 && tid == 0) set_err(a.err, kErrCache);
+    if (tid < NP) s_mask[tid] = tid < NQ ? a.front_mask[b * a.w + tid / G] : 0ull;
+    const int pc = pos >= 0 && pos < a.max_ctx ? pos : 0;
+    const float *cs_row = a.rope_cos + (size_t)pc * half, *sn_row = a.rope_sin + (size_t)pc * half;
+    // this step's rows of this rank's keys: rotated at the node's depth, into their own slots
+    for (int e = tid; e < a.w * (half / 4); e += kThr) {
+        const int j = e / (half / 4), q = e % (half / 4), slot = new0 + j;
+        if (slot < j0 || slot >= j1) continue;
+        const float *xk = a.qkv + (((size_t)b * a.w + j) * H + a.Hq + g) * D, *xv = xk + (size_t)a.Hkv * D;
+        const float4 x0 = __ldcg((const float4 *)xk + q), x1 = __ldcg((const float4 *)(xk + half) + q);
+        const float4 v0 = __ldcg((const float4 *)xv + 2 * q), v1 = __ldcg((const float4 *)xv + 2 * q + 1);
+        const float4 c = __ldg((const float4 *)cs_row + q), s = __ldg((const float4 *)sn_row + q);
+        const size_t o = (((size_t)b * a.Hkv + g) * a.max_ctx + slot) * D;
+        uint16_t *kc = (uint16_t *)a.k_cache + o, *vc = (uint16_t *)a.v_cache + o;
+        store4(kc + 4 * q, x0.x * c.x - x1.x * s.x, x0.y * c.y - x1.y * s.y, x0.z * c.z - x1.z * s.z, x0.w * c.w - x1.w * s.w);
+        store4(kc + half + 4 * q, x1.x * c.x + x0.x * s.x, x1.y * c.y + x0.y * s.y, x1.z * c.z + x0.z * s.z,
+               x1.w * c.w + x0.w * s.w);
+        store4(vc + 8 * q, v0.x, v0.y, v0.z, v0.w);
+        store4(vc + 8 * q + 4, v1.x, v1.y, v1.z, v1.w);
+    }
+    // queries, rotated, in log2 units (log2(e) / sqrt(D)), as bf16 hi + lo
+    const float scale = 1.4426950408889634f / sqrtf((float)D);
+    for (int e = tid; e < NP * (half / 2); e += kThr) {
+        const int pr = e / (half / 2), q = e % (half / 2);
+        uint32_t h0 = 0, l0 = 0, h1 = 0, l1 = 0;
+        if (pr < NQ) {
+            const float *x = a.qkv + (((size_t)b * a.w + pr / G) * H + g * G + pr % G) * D;
+            const float2 x0 = __ldcg((const float2 *)x + q), x1 = __ldcg((const float2 *)(x + half) + q);
+            const float2 c = __ldg((const float2 *)cs_row + q), s = __ldg((const float2 *)sn_row + q);
+            split2((x0.x * c.x - x1.x * s.x) * scale, (x0.y * c.y - x1.y * s.y) * scale, h0, l0);
+            split2((x1.x * c.x + x0.x * s.x) * scale, (x1.y * c.y + x0.y * s.y) * scale, h1, l1);
+        }
+        qh[pr * QW + q] = h0;
+        ql[pr * QW + q] = l0;
+        qh[pr * QW + half / 2 + q] = h1;
+        ql[pr * QW + half / 2 + q] = l1;
+    }
+    // the async proxy reads rows this kernel just wrote: order those writes first
+    asm volatile("fence.proxy.async.global;" ::: "memory");
+    __syncthreads();
+
+    // a warp's state: pairs p0 = 8 nt + 2 (lane % 4), p0 + 1; O^T dims 16 t + lane / 4 (+ 8)
+    bool dead = false;
+    float mx[NTN][2], sm[NTN][2], o[NTN][NT][4];
+#pragma unroll
+    for (int nt = 0; nt < NTN; ++nt) {
+        mx[nt][0] = mx[nt][1] = -INFINITY;
+        sm[nt][0] = sm[nt][1] = 0.f;
+#pragma unroll
+        for (int t = 0; t < NT; ++t) o[nt][t][0] = o[nt][t][1] = o[nt][t][2] = o[nt][t][3] = 0.f;
+    }
+    if (warp == W) {
+        // ---------------------------------------------------------------- producer
+        if (producer) {
+            int issued = pre;
+            for (int i = pre; i < nst && !dead; ++i) {
+                if (i >= kTaStages) {
+                    bool ok = false;
+                    const uint32_t par = (uint32_t)((i / kTaStages - 1) & 1);
+                    for (long it = 0; it < lim && !ok; ++it) ok = fa_try(&empty[i % kTaStages], par);
+                    if (!ok) {
+                        set_err(a.err, kErrTimeout);
+                        dead = true;
+                        break;
+                    }
+                }
+                load(i);
+                issued = i + 1;
+            }
+            if (!dead) prefetch_l2_share(a.pf_next, a.pf_next_bytes, r + CS * (g + a.Hkv * b), CS * a.Hkv * a.B);
+            for (int i = issued > kTaStages ? issued - kTaStages : 0; i < issued; ++i) {
+                bool ok = false;
+                for (long it = 0; it < kAttnWaitLimit && !ok; ++it)
+                    ok = fa_try(&full[i % kTaStages], (uint32_t)((i / kTaStages) & 1));
+                if (!ok) set_err(a.err, kErrTimeout);
+            }
+        }
+    } else {
+        // ---------------------------------------------------------------- compute warps
+        const int kr = 16 * warp, mi = lane >> 3;
+        const int qo = (lane >> 2) * QW + (lane & 3);
+        for (int i = 0; i < nst; ++i) {
+            const int s = i % kTaStages;
+            if (!dead && !ta_wait_warp(&full[s], (uint32_t)((i / kTaStages) & 1), lim)) {
+                if (lane == 0) set_err(a.err, kErrTimeout);
+                dead = true;
+            }
+            const int key0 = j0 + i * kC + kr, cnt = min(16, j1 - key0);
+            if (!dead && cnt > 0) {
+                const uint32_t kb = ring_s + (uint32_t)s * kStage, vb = kb + NH * kBox;
+                // value rows past the range: zero (their probabilities are, and 0 * NaN would not be)
+                if (cnt < 16) {
+                    for (int e = lane; e < (16 - cnt) * NH * 8; e += 32)
+                        asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};"
+                                     ::"r"(ta_piece<kC>(vb, kr + cnt + e / (NH * 8), e % (NH * 8))), "r"(0) : "memory");
+                    __syncwarp();
+                }
+                float sh[NTN][4] = {}, sl[NTN][4] = {};
+#pragma unroll
+                for (int ks = 0; ks < NT; ++ks) {
+                    uint32_t ka[4];
+                    ldsm_x4(ta_piece<kC>(kb, kr + (mi & 1) * 8 + (lane & 7), 2 * ks + (mi >> 1)), ka);
+#pragma unroll
+                    for (int nt = 0; nt < NTN; ++nt) {
+                        const int q = qo + nt * 8 * QW + 8 * ks;
+                        mma16816(sh[nt], ka, qh[q], qh[q + 4]);
+                        mma16816(sl[nt], ka, ql[q], ql[q + 4]);
+                    }
+                }
+                uint32_t pbh[NTN][2], pbl[NTN][2];
+#pragma unroll
+                for (int nt = 0; nt < NTN; ++nt) {
+                    float sv[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) sv[q] = sh[nt][q] + sl[nt][q];
+                    if (key0 + 16 > base || cnt < 16) {           // draft slots, or the range's end
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int key = (lane >> 2) + (q >> 1) * 8, off = key0 + key - base;
+                            const unsigned long long m = s_mask[nt * 8 + 2 * (lane & 3) + (q & 1)];
+                            const bool vis = key < cnt && (off < 0 || (off < kTreeMaskBits && ((m >> off) & 1ull)));
+                            if (!vis) sv[q] = -INFINITY;
+                        }
+                    }
+                    float c0 = fmaxf(sv[0], sv[2]), c1 = fmaxf(sv[1], sv[3]);
+#pragma unroll
+                    for (int off = 4; off < 32; off <<= 1) {
+                        c0 = fmaxf(c0, __shfl_xor_sync(0xFFFFFFFFu, c0, off));
+                        c1 = fmaxf(c1, __shfl_xor_sync(0xFFFFFFFFu, c1, off));
+                    }
+                    const float n0 = fmaxf(mx[nt][0], c0), n1 = fmaxf(mx[nt][1], c1);
+                    float p[4];
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float mq = (q & 1) ? n1 : n0;
+                        p[q] = (sv[q] == -INFINITY || mq == -INFINITY) ? 0.f : exp2f(sv[q] - mq);
+                    }
+                    if (__any_sync(0xFFFFFFFFu, n0 != mx[nt][0] || n1 != mx[nt][1])) {
+                        const float al0 = mx[nt][0] == -INFINITY ? 0.f : exp2f(mx[nt][0] - n0);
+                        const float al1 = mx[nt][1] == -INFINITY ? 0.f : exp2f(mx[nt][1] - n1);
+                        sm[nt][0] *= al0;
+                        sm[nt][1] *= al1;
+#pragma unroll
+                        for (int t = 0; t < NT; ++t) {
+                            o[nt][t][0] *= al0;
+                            o[nt][t][1] *= al1;
+                            o[nt][t][2] *= al0;
+                            o[nt][t][3] *= al1;
+                        }
+                    }
+                    sm[nt][0] += p[0] + p[2];
+                    sm[nt][1] += p[1] + p[3];
+                    mx[nt][0] = n0;
+                    mx[nt][1] = n1;
+                    uint32_t h01, l01, h23, l23;
+                    split2(p[0], p[1], h01, l01);
+                    split2(p[2], p[3], h23, l23);
+                    pbh[nt][0] = movm_t(h01);
+                    pbh[nt][1] = movm_t(h23);
+                    pbl[nt][0] = movm_t(l01);
+                    pbl[nt][1] = movm_t(l23);
+                }
+#pragma unroll
+                for (int t = 0; t < NT; ++t) {
+                    uint32_t va[4];
+                    ldsm_x4_t(ta_piece<kC>(vb, kr + (mi >> 1) * 8 + (lane & 7), 2 * t + (mi & 1)), va);
+#pragma unroll
+                    for (int nt = 0; nt < NTN; ++nt) {
+                        mma16816(o[nt][t], va, pbh[nt][0], pbh[nt][1]);
+                        mma16816(o[nt][t], va, pbl[nt][0], pbl[nt][1]);
+                    }
+                }
+                // zeros written above precede the next TMA write of this slot
+                if (cnt < 16) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
+            __syncwarp();
+            if (lane == 0 && !dead)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(sa(&empty[s])) : "memory");
+        }
+#pragma unroll
+        for (int nt = 0; nt < NTN; ++nt)
+#pragma unroll
+            for (int off = 4; off < 32; off <<= 1) {
+                sm[nt][0] += __shfl_xor_sync(0xFFFFFFFFu, sm[nt][0], off);
+                sm[nt][1] += __shfl_xor_sync(0xFFFFFFFFu, sm[nt][1], off);
+            }
+    }
+    __syncthreads();                                  // every copy landed, every warp done with ring and queries
+    if (warp < W) {
+#pragma unroll
+        for (int nt = 0; nt < NTN; ++nt) {
+            const int p0 = nt * 8 + 2 * (lane & 3), d0 = lane >> 2;
+            if (lane < 4) {
+                wm[warp * NP + p0] = mx[nt][0];
+                wm[warp * NP + p0 + 1] = mx[nt][1];
+                wl[warp * NP + p0] = sm[nt][0];
+                wl[warp * NP + p0 + 1] = sm[nt][1];
+            }
+            float *w0 = wo + (size_t)(warp * NP + p0) * D, *w1 = w0 + D;
+#pragma unroll
+            for (int t = 0; t < NT; ++t) {
+                w0[16 * t + d0] = o[nt][t][0];
+                w1[16 * t + d0] = o[nt][t][1];
+                w0[16 * t + d0 + 8] = o[nt][t][2];
+                w1[16 * t + d0 + 8] = o[nt][t][3];
+            }
+        }
+    }
+    __syncthreads();
+    // this rank's partial: the warps' states merged in warp order
+    for (int e = tid; e < NQ * D; e += kThr) {
+        const int pr = e / D, d = e % D;
+        float M = -INFINITY;
+#pragma unroll
+        for (int w = 0; w < W; ++w) M = fmaxf(M, wm[w * NP + pr]);
+        float num = 0.f, den = 0.f;
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+            const float mw = wm[w * NP + pr];
+            const float f = mw == -INFINITY ? 0.f : exp2f(mw - M);
+            den = fmaf(f, wl[w * NP + pr], den);
+            num = fmaf(f, wo[(size_t)(w * NP + pr) * D + d], num);
+        }
+        po[e] = num;
+        if (d == 0) {
+            pm[pr] = M;
+            pl[pr] = den;
+        }
+    }
+    cluster_sync_all();
+    // rank r combines its slice of the outputs from every rank, in rank order
+    const int n_out = NQ * D, e0 = (int)((long)r * n_out / CS), e1 = (int)((long)(r + 1) * n_out / CS);
+    for (int e = e0 + tid; e < e1; e += kThr) {
+        constexpr int kRanks = 8;
+        const int pr = e / D;
+        float mq[kRanks], lq[kRanks], oq[kRanks];
+#pragma unroll
+        for (int q = 0; q < kRanks; ++q) {
+            const bool in = q < CS;
+            mq[q] = in ? dsmem_ld(pm + pr, (uint32_t)q) : -INFINITY;
+            lq[q] = in ? dsmem_ld(pl + pr, (uint32_t)q) : 0.f;
+            oq[q] = in ? dsmem_ld(po + e, (uint32_t)q) : 0.f;
+        }
+        float M = -INFINITY;
+#pragma unroll
+        for (int q = 0; q < kRanks; ++q) M = fmaxf(M, mq[q]);
+        float num = 0.f, den = 0.f;
+#pragma unroll
+        for (int q = 0; q < kRanks; ++q) {
+            const float w = mq[q] == -INFINITY ? 0.f : exp2f(mq[q] - M);
+            den = fmaf(w, lq[q], den);
+            num = fmaf(w, oq[q], num);
+        }
+        uint16_t *out = (uint16_t *)a.o_out + (((size_t)b * a.w + pr / G) * a.Hq + g * G + pr % G) * D;
+        out[e % D] = f32_to_bf16(den > 0.f ? num / den : 0.f);
+    }
+    cluster_sync_all();
+}
+
+template <int D, int NTN>
+constexpr size_t tree_cl_smem() {
+    return 1024 + (size_t)kTaStages * 2 * (D / 64) * TaCfg<8>::kC * 128 + (size_t)2 * 8 * NTN * (D / 2 + 4) * 4 +
+           (size_t)2 * 8 * NTN * 4;
+}
+static_assert((size_t)(8 * 32 * 128 + 2 * 8 * 32) * 4 <= (size_t)kTaStages * 2 * 2 * TaCfg<8>::kC * 128 &&
+                  (size_t)(8 * 32 * 64 + 2 * 8 * 32) * 4 <= (size_t)kTaStages * 2 * TaCfg<8>::kC * 128,
+              "the warps' states fit in the ring");
+
 template <int D, int W>
 constexpr size_t fused_tc_smem() {
     return 1024 + (size_t)kTaStages * 2 * (D / 64) * TaCfg<W>::kC * 128 + (size_t)2 * 8 * D * 4 + 16 * 4;
@@ -1125,16 +1477,16 @@ size_t fused_smem(int G) {
 static_assert(kFusedThreads % 128 == 0, "score pass maps threads to (key, head group)");
 
 template <typename Kern, typename... Args>
-cudaError_t launch_cluster(Kern k, size_t smem, int threads, const FusedAttnArgs &a, cudaStream_t s, bool pdl,
+cudaError_t launch_cluster(Kern k, size_t smem, int threads, int cs, int Hkv, int B, cudaStream_t s, bool pdl,
                            Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(a.cs, a.Hkv, a.B);
+    cfg.gridDim = dim3(cs, Hkv, B);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = s;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = a.cs;
+    attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1150,13 +1502,44 @@ cudaError_t launch_fused_t(const FusedAttnArgs &a, cudaStream_t s, bool pdl, con
     if constexpr (sizeof(WT) == 2) {
         if (tk && tv && a.Hq / a.Hkv <= 8) {
             if (a.warps == 4)
-                return launch_cluster(fused_attention_tc_kernel<D, 4>, fused_tc_smem<D, 4>(), TaCfg<4>::kThreads, a, s,
-                                      pdl, a, *tk, *tv);
-            return launch_cluster(fused_attention_tc_kernel<D, 8>, fused_tc_smem<D, 8>(), TaCfg<8>::kThreads, a, s,
-                                  pdl, a, *tk, *tv);
+                return launch_cluster(fused_attention_tc_kernel<D, 4>, fused_tc_smem<D, 4>(), TaCfg<4>::kThreads, a.cs,
+                                      a.Hkv, a.B, s, pdl, a, *tk, *tv);
+            return launch_cluster(fused_attention_tc_kernel<D, 8>, fused_tc_smem<D, 8>(), TaCfg<8>::kThreads, a.cs,
+                                  a.Hkv, a.B, s, pdl, a, *tk, *tv);
         }
     }
-    return launch_cluster(fused_attention_kernel<WT, D>, fused_smem<WT, D>(a.Hq / a.Hkv), kFusedThreads, a, s, pdl, a);
+    return launch_cluster(fused_attention_kernel<WT, D>, fused_smem<WT, D>(a.Hq / a.Hkv), kFusedThreads, a.cs, a.Hkv, a.B, s, pdl,
+                          a);
+}
+
+template <int D, int NTN>
+cudaError_t launch_tree_cl(const TreeArgs &a, int cs, const CUtensorMap &tk, const CUtensorMap &tv, cudaStream_t s, bool pdl) {
+    return launch_cluster(tree_attention_cluster_kernel<D, NTN>, tree_cl_smem<D, NTN>(), TaCfg<8>::kThreads, cs, a.Hkv,
+                          a.B, s, pdl, a, tk, tv);
+}
+template <int D>
+cudaError_t launch_tree_cl_d(const TreeArgs &a, int cs, const CUtensorMap &tk, const CUtensorMap &tv, cudaStream_t s, bool pdl) {
+    switch ((a.w * (a.Hq / a.Hkv) + 7) / 8) {
+        case 1: return launch_tree_cl<D, 1>(a, cs, tk, tv, s, pdl);
+        case 2: return launch_tree_cl<D, 2>(a, cs, tk, tv, s, pdl);
+        case 3: return launch_tree_cl<D, 3>(a, cs, tk, tv, s, pdl);
+        case 4: return launch_tree_cl<D, 4>(a, cs, tk, tv, s, pdl);
+    }
+    return cudaErrorInvalidValue;
+}
+template <int D, int NTN>
+cudaError_t tree_cl_attr() {
+    static_assert(tree_cl_smem<D, NTN>() + 512 <= (size_t)227 * 1024, "tree attention shared memory");
+    return cudaFuncSetAttribute(tree_attention_cluster_kernel<D, NTN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)tree_cl_smem<D, NTN>());
+}
+template <int D>
+cudaError_t tree_cl_attrs() {
+    cudaError_t e = tree_cl_attr<D, 1>();
+    if (e == cudaSuccess) e = tree_cl_attr<D, 2>();
+    if (e == cudaSuccess) e = tree_cl_attr<D, 3>();
+    if (e == cudaSuccess) e = tree_cl_attr<D, 4>();
+    return e;
 }
 
 // Clusters of 16 are a non-portable size: allowed only where the occupancy
@@ -1257,6 +1640,14 @@ size_t attention_smem_bytes(bool bf16, int D, int chunk, int G, int splits) {
 }
 
 int fused_attention_chunk() { return kTaBoxRows; }
+
+cudaError_t prepare_tree_cluster_attention(int D) { return D == 64 ? tree_cl_attrs<64>() : tree_cl_attrs<128>(); }
+
+cudaError_t launch_tree_cluster_attention(const TreeArgs &a, int cs, const CUtensorMap &tk, const CUtensorMap &tv,
+                                          cudaStream_t s, bool pdl) {
+    if (cs < 1 || cs > 8) return cudaErrorInvalidValue;
+    return a.D == 64 ? launch_tree_cl_d<64>(a, cs, tk, tv, s, pdl) : launch_tree_cl_d<128>(a, cs, tk, tv, s, pdl);
+}
 
 cudaError_t launch_fused_attention(const FusedAttnArgs &a, bool bf16, cudaStream_t s, bool pdl,
                                    const CUtensorMap *tk, const CUtensorMap *tv) {

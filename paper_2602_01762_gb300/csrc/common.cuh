@@ -481,6 +481,7 @@ struct TreeArgs {
     int *attn_ctr;                    // [B, Hkv] (left at zero)
     void *o_out;                      // [B*w, Hq*D] wtype
     int chunk, splits;
+    int wait_polls;                   // see wait_bound
     // the O projection's weights, requested into L2 as in GemvArgs
     const void *pf_next;
     long long pf_next_bytes;
@@ -496,7 +497,7 @@ struct AcceptTreeArgs {
     int B, n_nodes, K;
 };
 size_t tree_attention_smem_bytes(bool bf16, int D, int chunk, int G, int w, int splits);
-cudaError_t prepare_tree_kernels(bool bf16, int D, int chunk, int G, int w, int splits, int max_ctx);
+cudaError_t prepare_tree_kernels(bool bf16, int D, int chunk, int G, int w, int splits);
 cudaError_t launch_tree_gather(const TreeArgs &a, bool bf16, cudaStream_t s, bool pdl);
 cudaError_t launch_tree_attention(const TreeArgs &a, bool bf16, cudaStream_t s, bool pdl);
 cudaError_t launch_tree_lse(const TreeArgs &a, cudaStream_t s, bool pdl);
@@ -562,6 +563,12 @@ int fused_attention_chunk();
 // given, the CUDA-core kernel otherwise.
 cudaError_t launch_fused_attention(const FusedAttnArgs &a, bool bf16, cudaStream_t s, bool pdl,
                                    const CUtensorMap *tk, const CUtensorMap *tv);
+// Tree attention over bf16 caches with at most kTreeClusterPairs row-head pairs
+// (w * G): one cluster of cs <= 8 CTAs per (sequence, KV head).
+constexpr int kTreeClusterPairs = 32;
+cudaError_t prepare_tree_cluster_attention(int D);
+cudaError_t launch_tree_cluster_attention(const TreeArgs &a, int cs, const CUtensorMap &tk, const CUtensorMap &tv,
+                                          cudaStream_t s, bool pdl);
 size_t attention_smem_bytes(bool bf16, int D, int chunk, int G, int splits);
 
 // Launch with optional programmatic stream serialization.

@@ -322,11 +322,14 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
         return launch_gemv(g, c->bf16, grid, s, pdl_here);
     };
 
-    // the caches as TMA tensor maps for the tensor-core attention kernel
+    // the caches as TMA tensor maps for the tensor-core attention kernels
     CUtensorMap tmk, tmv;
-    const bool cache_maps = c->attn_fused && c->attn_tc && c->bf16 && c->tc_ready &&
-                            make_cache_map(&tmk, r.k_cache, r.B * Hkv, f.max_ctx, D, fused_attention_chunk()) == cudaSuccess &&
-                            make_cache_map(&tmv, r.v_cache, r.B * Hkv, f.max_ctx, D, fused_attention_chunk()) == cudaSuccess;
+    const bool chain_maps = c->attn_fused && c->attn_tc;
+    const bool maps = (chain_maps || r.tree_w > 0) && c->bf16 && c->tc_ready &&
+                      make_cache_map(&tmk, r.k_cache, r.B * Hkv, f.max_ctx, D, fused_attention_chunk()) == cudaSuccess &&
+                      make_cache_map(&tmv, r.v_cache, r.B * Hkv, f.max_ctx, D, fused_attention_chunk()) == cudaSuccess;
+    const bool cache_maps = chain_maps && maps;
+    const bool tree_cluster = maps && r.tree_w > 0 && r.tree_w * (Hq / Hkv) <= kTreeClusterPairs;
 
     // tree drafting: w rows per sequence from step 2 on
     const bool tree = r.tree_w > 0;
@@ -375,6 +378,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
         ta.o_out = c->o_buf;
         ta.chunk = c->attn_chunk;
         ta.splits = c->attn_splits;
+        ta.wait_polls = c->wait_polls;
         ta.tree_tokens = r.tree.tokens;
         ta.tree_parents = r.tree.parents;
         ta.tree_depths = r.tree.depths;
@@ -572,7 +576,10 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             const auto n = pf(c->steps[k - 1].w_o, (size_t)d * Hq * D);
             ta.pf_next = n.first;
             ta.pf_next_bytes = n.second;
-            e = launch_tree_attention(ta, c->bf16, s, pdl);
+            int cs = std::min(c->attn_max_cs, 8);
+            while (cs > 1 && (long long)r.B * Hkv * cs > (long long)c->attn_ctas_per_sm * c->sms) cs /= 2;
+            e = tree_cluster ? launch_tree_cluster_attention(ta, cs, tmk, tmv, s, pdl)
+                             : launch_tree_attention(ta, c->bf16, s, pdl);
             after(3);
             if (e != cudaSuccess) break;
         } else if (c->attn_fused) {
@@ -949,7 +956,8 @@ prism_status prism_create(const prism_config *cfg, int32_t device, prism_ctx **o
             delete c;
             return fail(nullptr, PRISM_ERR_INVALID_ARG, "max_ctx too large for the tree attention combine");
         }
-        e = prepare_tree_kernels(c->bf16, D, c->attn_chunk, Hq / Hkv, (int)TW, c->attn_splits, f.max_ctx);
+        e = prepare_tree_kernels(c->bf16, D, c->attn_chunk, Hq / Hkv, (int)TW, c->attn_splits);
+        if (e == cudaSuccess && c->bf16) e = prepare_tree_cluster_attention(D);
     }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&c->cap_stream, cudaStreamNonBlocking);
     if (e != cudaSuccess) {

@@ -12,15 +12,15 @@
 // of the round.  The kernels this file adds:
 //   tree_gather_kernel     fusion input row [E(token); round(h^ of the row
 //                          that emitted the token)];
-//   tree_attention_tc_kernel / tree_attention_kernel
-//                          rotary embedding at the node's depth, K/V appended
+//   tree_attention_kernel  rotary embedding at the node's depth, K/V appended
 //                          at the node's own cache slot L + n + (k - 2) w + j,
 //                          and split-KV attention over the committed rows
 //                          [0, L+n) plus the draft slots in the row's 64-bit
 //                          ancestor mask, all w rows of a sequence against one
 //                          staged chunk of keys, last-CTA merge in split order
-//                          (tensor cores for bf16 caches with w * G <= 16
-//                          row-head pairs, CUDA cores otherwise);
+//                          on the CUDA cores (bf16 caches with at most
+//                          kTreeClusterPairs row-head pairs take the cluster
+//                          kernel of attention.cu);
 //   tree_lse_kernel        log-sum-exp of every row's logits; the last row of
 //                          each sequence to finish then scores the candidates,
 //                          picks the next frontier and, after the last step,
@@ -296,7 +296,7 @@ __device__ __forceinline__ bool tree_visible(int p, int base, unsigned long long
 
 constexpr int kTreeAttnThreads = 512;   // 16 warps: one (row, query head) pair each when w * G = 16
 
-// CUDA-core kernel (fp32 caches, or more than 16 row-head pairs).  Grid
+// CUDA-core kernel (fp32 caches, or more than kTreeClusterPairs row-head pairs).  Grid
 // (splits, Hkv, B); CTA (s, g, b) stages keys [s C, s C + C) of KV head g once
 // and each warp scores them against one (row, query head) pair at a time.
 template <typename WT, int D>
@@ -383,229 +383,6 @@ __global__ void __launch_bounds__(kTreeAttnThreads) tree_attention_kernel(const 
         }
     }
     tree_merge_splits<WT, D>(a, b, g, ws, &s_last);
-}
-
-// ------------------------------------------------------------------ attention on tensor cores
-
-// bf16 caches with at most 16 row-head pairs (w * G <= 16).  CTA (s, g, b)
-// stages kTcChunk keys as above; compute warp w takes keys 16w .. 16w + 15 in
-// the M dimension of mma.sync.m16n8k16 with the pairs in N (one or two n8
-// tiles).  S^T = K q^T with each query (rotated, times 1/sqrt(D)) split into a
-// bf16 hi + lo pair (two MMAs: operand error near 2^-17, K exact); the warp's
-// softmax per pair over its 16 keys; P^T from the S^T tile by movmatrix (the
-// accumulator layout of S^T is the B-fragment layout of P^T, transposed), also
-// split hi + lo; O^T += V^T P^T with V^T read by a transposing ldmatrix.  The
-// warps' (max, sum, O) merge in shared memory into the CTA's split partial;
-// the splits then merge as in the CUDA-core kernel.
-constexpr int kTcWarps = 8;
-constexpr int kTcChunk = kTcWarps * 16;
-constexpr int kTcMaxPairs = 16;
-
-__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t addr, uint32_t (&r)[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ uint32_t movm_t(uint32_t x) {
-    uint32_t y;
-    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(y) : "r"(x));
-    return y;
-}
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, "
-                 "{%8, %9}, {%0, %1, %2, %3};"
-                 : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// bf16 hi / lo parts of two floats, packed (low half = first element).
-__device__ __forceinline__ void split2(float x, float y, uint32_t &hi, uint32_t &lo) {
-    const uint16_t hx = f32_to_bf16(x), hy = f32_to_bf16(y);
-    hi = (uint32_t)hx | ((uint32_t)hy << 16);
-    lo = (uint32_t)f32_to_bf16(x - bf16_to_f32(hx)) | ((uint32_t)f32_to_bf16(y - bf16_to_f32(hy)) << 16);
-}
-
-template <int D>
-__global__ void __launch_bounds__(kTcWarps * 32) tree_attention_tc_kernel(const TreeArgs a) {
-    constexpr int RS = D + 8;                 // bf16 row stride: 16-byte rows, conflict-free ldmatrix
-    constexpr int NT = D / 16;                // 16-dim tiles
-    constexpr int PS = D + 4;
-    constexpr int QS = D + 8;                 // query row stride: at most 2-way bank conflicts in the B loads
-    extern __shared__ __align__(16) uint8_t smem_raw[];
-    __shared__ int s_last;
-    __shared__ unsigned long long s_mask[kTreeMaxWidth];
-    uint16_t *Ks = (uint16_t *)smem_raw;
-    uint16_t *Vs = Ks + (size_t)kTcChunk * RS;
-    float *qs = (float *)(Vs + (size_t)kTcChunk * RS);  // [16][QS] scaled queries, pairs >= NQ zero
-    float *wm = qs + kTcMaxPairs * QS;                  // [warp][16]
-    float *wl = wm + kTcWarps * kTcMaxPairs;            // [warp][16]
-    float *ws = wl + kTcWarps * kTcMaxPairs;            // [16][splits]
-    float *wo = (float *)smem_raw;                      // [warp][16][D], after the keys are consumed
-    const int s = blockIdx.x, g = blockIdx.y, b = blockIdx.z;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int G = a.Hq / a.Hkv, NQ = a.w * G;
-
-    pdl_trigger();
-
-    const int n = tree_n(a, b), L = a.kv_len[b];
-    const int base = L + n;
-    int PE = base + (a.step - 1) * a.w;
-    if (PE > a.max_ctx) PE = a.max_ctx;
-    const int j0 = s * kTcChunk;
-    int nk = PE - j0 < kTcChunk ? PE - j0 : kTcChunk;
-    if (L < 0) nk = 0;
-    const int ncom = nk > 0 ? tree_stage_committed<uint16_t, D, RS>(a, b, g, j0, nk, L, Ks, Vs) : 0;
-    pdl_wait();
-    if (s == 0 && g == 0 && tid == 0 && (L < 0 || base + (a.step - 1) * a.w > a.max_ctx)) set_err(a.err, kErrCache);
-    if (tid < a.w) s_mask[tid] = a.front_mask[b * a.w + tid];
-    for (int e = tid; e < (kTcMaxPairs - NQ) * QS; e += blockDim.x) qs[NQ * QS + e] = 0.f;
-    if (nk > 0) {
-        tree_stage<uint16_t, D, RS, QS>(a, b, g, j0, nk, base, Ks, Vs, qs, 1.0f / sqrtf((float)D), ncom);
-        // rows past the chunk's keys: zero (their probabilities are 0, and 0 * NaN would not be)
-        for (int e = tid; e < (kTcChunk - nk) * (D / 8); e += blockDim.x) {
-            const int r = nk + e / (D / 8), c = e % (D / 8);
-            *(uint4 *)(Ks + (size_t)r * RS + c * 8) = make_uint4(0, 0, 0, 0);
-            *(uint4 *)(Vs + (size_t)r * RS + c * 8) = make_uint4(0, 0, 0, 0);
-        }
-    }
-    cp_async_wait_all();
-    __syncthreads();
-    // this CTA's keys are in: its share of the next kernel's weights into L2
-    if (tid == 0)
-        prefetch_l2_share(a.pf_next, a.pf_next_bytes, s + a.splits * (g + a.Hkv * b), a.splits * a.Hkv * a.B);
-
-    // warp state: pairs nt * 8 + 2 (lane % 4) + {0, 1}; O^T dims 16 t + lane / 4 (+ 8)
-    const int kr = 16 * warp;
-    const int cnt = nk - kr;                  // keys of this warp (may be <= 0)
-    const int ntn = (NQ + 7) / 8;
-    float mx[2][2], sm[2][2], o[2][NT][4];
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-        mx[nt][0] = mx[nt][1] = -INFINITY;
-        sm[nt][0] = sm[nt][1] = 0.f;
-#pragma unroll
-        for (int t = 0; t < NT; ++t) o[nt][t][0] = o[nt][t][1] = o[nt][t][2] = o[nt][t][3] = 0.f;
-    }
-    if (cnt > 0) {
-        const uint32_t kb = (uint32_t)__cvta_generic_to_shared(Ks), vb = (uint32_t)__cvta_generic_to_shared(Vs);
-        const int mi = lane >> 3;
-        float sh[2][4], sl[2][4];
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) sh[nt][q] = sl[nt][q] = 0.f;
-#pragma unroll
-        for (int ks = 0; ks < NT; ++ks) {
-            uint32_t ka[4];
-            ldsm_x4(kb + (uint32_t)(((kr + (mi & 1) * 8 + (lane & 7)) * RS + 16 * ks + (mi >> 1) * 8) * 2), ka);
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                if (nt >= ntn) break;
-                uint32_t qh[2], ql[2];
-#pragma unroll
-                for (int u = 0; u < 2; ++u) {
-                    const float *src = qs + (nt * 8 + (lane >> 2)) * QS + 16 * ks + 2 * (lane & 3) + 8 * u;
-                    split2(src[0], src[1], qh[u], ql[u]);
-                }
-                mma16816(sh[nt], ka, qh[0], qh[1]);
-                mma16816(sl[nt], ka, ql[0], ql[1]);
-            }
-        }
-        uint32_t pbh[2][2], pbl[2][2];
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt) {
-            float sv[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int key = (lane >> 2) + (q >> 1) * 8, pr = nt * 8 + 2 * (lane & 3) + (q & 1);
-                const bool vis = key < cnt && pr < NQ && tree_visible(j0 + kr + key, base, s_mask[pr / G]);
-                sv[q] = vis ? sh[nt][q] + sl[nt][q] : -INFINITY;
-            }
-            // softmax per pair over the warp's 16 keys: lanes with equal lane % 4 share pairs
-            float c0 = fmaxf(sv[0], sv[2]), c1 = fmaxf(sv[1], sv[3]);
-#pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
-                c0 = fmaxf(c0, __shfl_xor_sync(0xFFFFFFFFu, c0, off));
-                c1 = fmaxf(c1, __shfl_xor_sync(0xFFFFFFFFu, c1, off));
-            }
-            mx[nt][0] = c0;
-            mx[nt][1] = c1;
-            float p[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const float mq = (q & 1) ? c1 : c0;
-                p[q] = sv[q] == -INFINITY ? 0.f : expf(sv[q] - mq);
-            }
-            sm[nt][0] = p[0] + p[2];
-            sm[nt][1] = p[1] + p[3];
-            uint32_t h01, l01, h23, l23;
-            split2(p[0], p[1], h01, l01);
-            split2(p[2], p[3], h23, l23);
-            pbh[nt][0] = movm_t(h01);
-            pbh[nt][1] = movm_t(h23);
-            pbl[nt][0] = movm_t(l01);
-            pbl[nt][1] = movm_t(l23);
-        }
-#pragma unroll
-        for (int t = 0; t < NT; ++t) {
-            uint32_t va[4];
-            ldsm_x4_t(vb + (uint32_t)(((kr + (mi >> 1) * 8 + (lane & 7)) * RS + 16 * t + (mi & 1) * 8) * 2), va);
-#pragma unroll
-            for (int nt = 0; nt < 2; ++nt) {
-                if (nt >= ntn) break;
-                mma16816(o[nt][t], va, pbh[nt][0], pbh[nt][1]);
-                mma16816(o[nt][t], va, pbl[nt][0], pbl[nt][1]);
-            }
-        }
-#pragma unroll
-        for (int nt = 0; nt < 2; ++nt)
-#pragma unroll
-            for (int off = 4; off < 32; off <<= 1) {
-                sm[nt][0] += __shfl_xor_sync(0xFFFFFFFFu, sm[nt][0], off);
-                sm[nt][1] += __shfl_xor_sync(0xFFFFFFFFu, sm[nt][1], off);
-            }
-    }
-    __syncthreads();                          // every warp is done with K and V: wo may overwrite them
-#pragma unroll
-    for (int nt = 0; nt < 2; ++nt) {
-        const int p0 = nt * 8 + 2 * (lane & 3);
-        if (lane < 4) {
-            wm[warp * kTcMaxPairs + p0] = mx[nt][0];
-            wm[warp * kTcMaxPairs + p0 + 1] = mx[nt][1];
-            wl[warp * kTcMaxPairs + p0] = sm[nt][0];
-            wl[warp * kTcMaxPairs + p0 + 1] = sm[nt][1];
-        }
-#pragma unroll
-        for (int t = 0; t < NT; ++t)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int d = 16 * t + (lane >> 2) + (q >> 1) * 8, pr = p0 + (q & 1);
-                wo[((size_t)warp * kTcMaxPairs + pr) * D + d] = o[nt][t][q];
-            }
-    }
-    __syncthreads();
-    // the CTA's partial of each pair: warps merged in warp order
-    for (int e = tid; e < NQ * D; e += blockDim.x) {
-        const int pr = e / D, d = e % D;
-        float M = -INFINITY;
-#pragma unroll
-        for (int w = 0; w < kTcWarps; ++w) M = fmaxf(M, wm[w * kTcMaxPairs + pr]);
-        float acc = 0.f, den = 0.f;
-#pragma unroll
-        for (int w = 0; w < kTcWarps; ++w) {
-            const float lw = wl[w * kTcMaxPairs + pr];
-            const float wt = lw > 0.f ? expf(wm[w * kTcMaxPairs + pr] - M) : 0.f;
-            acc = fmaf(wt, wo[((size_t)w * kTcMaxPairs + pr) * D + d], acc);
-            den = fmaf(wt, lw, den);
-        }
-        const int j = pr / G, hl = pr % G, t = b * a.w + j;
-        float *part = a.attn_part + (((size_t)t * a.Hq + (size_t)g * G + hl) * a.splits + s) * PS;
-        part[d] = acc;
-        if (d == 0) { part[D] = M; part[D + 1] = den; }
-    }
-    tree_merge_splits<uint16_t, D>(a, b, g, ws, &s_last);
 }
 
 // ------------------------------------------------------------------ selection
@@ -886,36 +663,15 @@ size_t tree_attn_smem(int chunk, int G, int w, int splits) {
     return 2 * (size_t)chunk * RS * sizeof(WT) + ((size_t)NQ * D + (size_t)NQ * chunk + (size_t)NQ * splits) * 4;
 }
 
-template <int D>
-size_t tree_attn_tc_smem(int splits) {
-    return 2 * (size_t)kTcChunk * (D + 8) * 2 + ((size_t)kTcMaxPairs * (D + 8) + 2 * kTcWarps * kTcMaxPairs +
-                                                 (size_t)kTcMaxPairs * splits) * 4;
-}
-
-// the tensor-core kernel's split count (kTcChunk keys per CTA)
-int tc_splits(int max_ctx) { return (max_ctx + kTcChunk - 1) / kTcChunk; }
-
 template <typename WT, int D>
 cudaError_t launch_tree_attn_t(const TreeArgs &args, cudaStream_t s, bool pdl) {
-    if (sizeof(WT) == 2 && args.w * (args.Hq / args.Hkv) <= kTcMaxPairs && tc_splits(args.max_ctx) <= 256) {
-        TreeArgs a = args;
-        a.chunk = kTcChunk;
-        a.splits = tc_splits(a.max_ctx);
-        return launch_k(tree_attention_tc_kernel<D>, dim3(a.splits, a.Hkv, a.B), dim3(kTcWarps * 32),
-                        tree_attn_tc_smem<D>(a.splits), s, pdl, a);
-    }
     const size_t smem = tree_attn_smem<WT, D>(args.chunk, args.Hq / args.Hkv, args.w, args.splits);
     return launch_k(tree_attention_kernel<WT, D>, dim3(args.splits, args.Hkv, args.B), dim3(kTreeAttnThreads), smem,
                     s, pdl, args);
 }
 
 template <typename WT, int D>
-cudaError_t prepare_tree_attn_t(int chunk, int G, int w, int splits, int max_ctx) {
-    if (sizeof(WT) == 2 && tc_splits(max_ctx) <= 256) {
-        cudaError_t e = cudaFuncSetAttribute(tree_attention_tc_kernel<D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)tree_attn_tc_smem<D>(tc_splits(max_ctx)));
-        if (e != cudaSuccess) return e;
-    }
+cudaError_t prepare_tree_attn_t(int chunk, int G, int w, int splits) {
     const size_t smem = tree_attn_smem<WT, D>(chunk, G, w, splits);
     return cudaFuncSetAttribute(tree_attention_kernel<WT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
@@ -927,11 +683,11 @@ size_t tree_attention_smem_bytes(bool bf16, int D, int chunk, int G, int w, int 
     return D == 64 ? tree_attn_smem<float, 64>(chunk, G, w, splits) : tree_attn_smem<float, 128>(chunk, G, w, splits);
 }
 
-cudaError_t prepare_tree_kernels(bool bf16, int D, int chunk, int G, int w, int splits, int max_ctx) {
-    if (bf16) return D == 64 ? prepare_tree_attn_t<uint16_t, 64>(chunk, G, w, splits, max_ctx)
-                             : prepare_tree_attn_t<uint16_t, 128>(chunk, G, w, splits, max_ctx);
-    return D == 64 ? prepare_tree_attn_t<float, 64>(chunk, G, w, splits, max_ctx)
-                   : prepare_tree_attn_t<float, 128>(chunk, G, w, splits, max_ctx);
+cudaError_t prepare_tree_kernels(bool bf16, int D, int chunk, int G, int w, int splits) {
+    if (bf16) return D == 64 ? prepare_tree_attn_t<uint16_t, 64>(chunk, G, w, splits)
+                             : prepare_tree_attn_t<uint16_t, 128>(chunk, G, w, splits);
+    return D == 64 ? prepare_tree_attn_t<float, 64>(chunk, G, w, splits)
+                   : prepare_tree_attn_t<float, 128>(chunk, G, w, splits);
 }
 
 cudaError_t launch_tree_gather(const TreeArgs &a, bool bf16, cudaStream_t s, bool pdl) {

@@ -26,7 +26,7 @@
 //     chunk of units, publishes one list per row, and topk_merge_kernel joins
 //     the CTAs' lists (the last CTA did that alone, with dependent loads).
 // A round of three sequences at hidden 1024, vocabulary 32000, K 4 (743 MB of
-// weights): 741 us on the ring kernel that took fp32 before, 342 us here.
+// weights): 741 us on the ring kernel that took fp32 before, 327 us here.
 #include <algorithm>
 
 #include "common.cuh"
@@ -49,6 +49,7 @@ struct F32Plan {
     int seg;       // warps that share an item's contraction
     int stages;    // ring stages per warp: 6, 4 or 2
     int chunk;     // LM head: items per selection chunk
+    int prefetch;  // 1: request the next layer's first weights into L2
 };
 
 __device__ __forceinline__ void cp_async16(uint32_t dst, const void *src, uint64_t pol) {
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
             c0 = c1;
         } while (c0 < i1);
     }
-    if (threadIdx.x == 0) prefetch_l2_share(a.pf_next, a.pf_next_bytes, blockIdx.x, gridDim.x);
+    if (p.prefetch && threadIdx.x == 0) prefetch_l2_share(a.pf_next, a.pf_next_bytes, blockIdx.x, gridDim.x);
 }
 
 template <int TN>
@@ -352,6 +353,9 @@ bool f32_plan(const GemvArgs &a, int grid, F32Plan &p, size_t &smem) {
     const int n_items = (a.n_units + UI - 1) / UI, per_cta = (n_items + grid - 1) / grid;
     // a CTA's weights in bytes: below this two 8-warp CTAs to an SM
     const bool small = (size_t)per_cta * kMR * a.kin * 4 < 384 * 1024;
+    // beside such CTAs the next layer's own rings are already filling: requests
+    // for its first bytes only delay them (339 us a round with, 327 without, three sequences as above)
+    p.prefetch = !small;
     p.tn = a.T <= 1 ? 1 : a.T <= 2 ? 2 : a.T <= 4 ? 4 : 8;
     p.tg = a.T <= 8 ? 1 : a.T <= 16 ? 2 : 4;
     for (;;) {

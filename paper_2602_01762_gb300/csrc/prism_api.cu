@@ -331,6 +331,18 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
     const bool cache_maps = chain_maps && maps;
     const bool tree_cluster = maps && r.tree_w > 0 && r.tree_w * (Hq / Hkv) <= kTreeClusterPairs;
 
+    // CTAs per (sequence, KV head) of the attention kernels: halved while they
+    // exceed attn_ctas_per_sm per SM, and while half as many already take the
+    // whole cache in one stage each: a cluster's merge then costs more than its
+    // CTAs save (tiny drafter, batch 8, contexts 64 to 200: 177 us a round in
+    // clusters of 8, 147 so; hidden 1024, batch 6, contexts to 400: 335 and 306)
+    auto attn_cluster = [&](int most, int stage_keys) {
+        int cs = most;
+        while (cs > 1 && ((long long)r.B * Hkv * cs > (long long)c->attn_ctas_per_sm * c->sms ||
+                          (long long)(cs / 2) * stage_keys >= f.max_ctx)) cs /= 2;
+        return cs;
+    };
+
     // tree drafting: w rows per sequence from step 2 on
     const bool tree = r.tree_w > 0;
     const int tw = tree ? r.tree_w : 1;
@@ -576,9 +588,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             const auto n = pf(c->steps[k - 1].w_o, (size_t)d * Hq * D);
             ta.pf_next = n.first;
             ta.pf_next_bytes = n.second;
-            int cs = std::min(c->attn_max_cs, 8);
-            while (cs > 1 && (long long)r.B * Hkv * cs > (long long)c->attn_ctas_per_sm * c->sms) cs /= 2;
-            e = tree_cluster ? launch_tree_cluster_attention(ta, cs, tmk, tmv, s, pdl)
+            e = tree_cluster ? launch_tree_cluster_attention(ta, attn_cluster(std::min(c->attn_max_cs, 8), 128), tmk, tmv, s, pdl)
                              : launch_tree_attention(ta, c->bf16, s, pdl);
             after(3);
             if (e != cudaSuccess) break;
@@ -601,8 +611,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             fa.Hkv = Hkv;
             fa.D = D;
             fa.max_ctx = f.max_ctx;
-            fa.cs = c->attn_max_cs;
-            while (fa.cs > 1 && (long long)r.B * Hkv * fa.cs > (long long)c->attn_ctas_per_sm * c->sms) fa.cs /= 2;
+            fa.cs = attn_cluster(c->attn_max_cs, c->bf16 ? 128 : 64);
             fa.err = c->err;
             fa.wait_polls = c->wait_polls;
             {

@@ -369,9 +369,11 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * per tile adds the sums itself; a greedy LM head other than that streamed
  * top-1 below (lm_stream) streams from max(this, 8) rows outside tree rounds), "attn_ctas_per_sm" (1..64, default 2: the fused attention
  * kernel's cluster size halves while batch x KV heads x cluster size exceeds
- * this many CTAs per SM), "gemv_cuda_core" (for projections
- * not on the tcgen05 kernel: 1, the default, the CUDA-core TMA-ring kernel;
- * 0: the warp-level mma.sync kernel), "attn_fused" (1, the default: RoPE,
+ * this many CTAs per SM, while half as many CTAs already take the whole cache
+ * (max_ctx) in one stage each, and, above 2, while the device cannot hold all
+ * clusters of that size at once), "gemv_cuda_core" (for projections
+ * not on the tcgen05 kernel, bf16: 1, the default, the CUDA-core TMA-ring
+ * kernel; 0: the warp-level mma.sync kernel), "attn_fused" (1, the default: RoPE,
  * KV append and attention run as one kernel, a cluster of up to 8 CTAs per
  * sequence and KV head merging through distributed shared memory; 0: a
  * RoPE/append kernel, then split-KV attention with a last-CTA merge),
@@ -380,8 +382,9 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * and PV with warp-level tensor-core MMAs; 0: the same fused computation on
  * CUDA cores), "attn_warps" (compute warps per CTA of that tensor-core
  * kernel: 8, stages of 128 keys, one CTA per SM; or 4, stages of 64 keys,
- * two CTAs per SM; 0, the default: 4 where one CTA per (sequence, KV head)
- * makes more CTAs than SMs but at most two per SM, else 8), "attn_lpt" (1,
+ * two CTAs per SM; 0, the default: 4 where the CTAs are more than the SMs,
+ * except clusters of two over caches of more than 3072 rows and several
+ * sequences, else 8), "attn_lpt" (1,
  * the default: where that kernel's CTAs make more than one wave but at most
  * two, the CTAs take the sequences in order of decreasing context length;
  * 0: in index order),
@@ -392,8 +395,9 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * testing the error path.  A wait that gives up sets the timeout bit and
  * the kernel winds down: it issues no more copies or MMAs, still waits
  * (with the built-in bound) for the copies and MMAs it has in flight, and
- * frees its tensor memory.  Covers the projection kernels and the fused
- * attention kernel),
+ * frees its tensor memory.  Covers the bf16 projection kernels, the fused
+ * attention kernel and the tree's attention kernel; the fp32 projections
+ * have no such waits),
  * "w_evict_first" (1, the default: the projection kernels load weight boxes
  * with an L2 evict-first cache policy, since each weight byte is read once
  * per step, so that the KV cache and the activations stay in L2; 0: the

@@ -1542,21 +1542,16 @@ cudaError_t tree_cl_attrs() {
     return e;
 }
 
-// Clusters of 16 are a non-portable size: allowed only where the occupancy
-// query confirms that `need` of them can be resident at once.
+// Clusters of cs CTAs of kernel k that the device holds at once (0: unknown).
 template <typename Kern>
-int max_cluster_for(Kern k, size_t smem, int threads, int need) {
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return 8;
-    }
+int clusters_resident(Kern k, size_t smem, int threads, int cs) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(16, 1, 1);
+    cfg.gridDim = dim3(cs, 1, 1);
     cfg.blockDim = dim3(threads);
     cfg.dynamicSmemBytes = smem;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 16;
+    attr[0].val.clusterDim.x = cs;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
@@ -1564,20 +1559,28 @@ int max_cluster_for(Kern k, size_t smem, int threads, int need) {
     int n = 0;
     if (cudaOccupancyMaxActiveClusters(&n, k, &cfg) != cudaSuccess) {
         cudaGetLastError();
-        return 8;
+        return 0;
     }
-    return n >= need ? 16 : 8;
+    return n;
+}
+// The cluster sizes the attention may take: clusters of 16, a non-portable
+// size, only where `need` of them can be resident at once.
+template <typename Kern>
+void cluster_limits(Kern k, size_t smem, int threads, int need, AttnClusters *c) {
+    const bool wide = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    if (!wide) cudaGetLastError();
+    c->most = wide && clusters_resident(k, smem, threads, 16) >= need ? 16 : 8;
+    for (int i = 0; i < 3; ++i) c->resident[i] = clusters_resident(k, smem, threads, 2 << i);
 }
 
 template <typename WT, int D>
-cudaError_t prepare_fused_t(int G, int need, int *max_cs) {
+cudaError_t prepare_fused_t(int G, int need, AttnClusters *cl) {
     // the CUDA-core kernel serves every cache type (and bf16 caches without
     // tensor maps); the tensor-core kernel bf16 caches with G <= 8
     if (G > 16 || fused_smem<WT, D>(G) > (size_t)200 * 1024) return cudaErrorInvalidValue;
     cudaError_t e = cudaFuncSetAttribute(fused_attention_kernel<WT, D>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          200 * 1024);
-    if (e == cudaSuccess && max_cs)
-        *max_cs = max_cluster_for(fused_attention_kernel<WT, D>, fused_smem<WT, D>(G), kFusedThreads, need);
+    if (e == cudaSuccess) cluster_limits(fused_attention_kernel<WT, D>, fused_smem<WT, D>(G), kFusedThreads, need, cl);
     if constexpr (sizeof(WT) == 2) {
         if (e == cudaSuccess && G <= 8) {
             static_assert(fused_tc_smem<D, 8>() <= (size_t)227 * 1024, "tensor-core attention shared memory");
@@ -1586,9 +1589,8 @@ cudaError_t prepare_fused_t(int G, int need, int *max_cs) {
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(fused_attention_tc_kernel<D, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)fused_tc_smem<D, 4>());
-            if (e == cudaSuccess && max_cs)
-                *max_cs = max_cluster_for(fused_attention_tc_kernel<D, 8>, fused_tc_smem<D, 8>(), TaCfg<8>::kThreads,
-                                          need);
+            if (e == cudaSuccess)
+                cluster_limits(fused_attention_tc_kernel<D, 8>, fused_tc_smem<D, 8>(), TaCfg<8>::kThreads, need, cl);
         }
     }
     return e;
@@ -1659,9 +1661,9 @@ cudaError_t launch_fused_attention(const FusedAttnArgs &a, bool bf16, cudaStream
                      : launch_fused_t<float, 128>(a, s, pdl, nullptr, nullptr);
 }
 
-cudaError_t prepare_fused_attention(bool bf16, int D, int G, int need, int *max_cs) {
-    if (bf16) return D == 64 ? prepare_fused_t<uint16_t, 64>(G, need, max_cs) : prepare_fused_t<uint16_t, 128>(G, need, max_cs);
-    return D == 64 ? prepare_fused_t<float, 64>(G, need, max_cs) : prepare_fused_t<float, 128>(G, need, max_cs);
+cudaError_t prepare_fused_attention(bool bf16, int D, int G, int need, AttnClusters *cl) {
+    if (bf16) return D == 64 ? prepare_fused_t<uint16_t, 64>(G, need, cl) : prepare_fused_t<uint16_t, 128>(G, need, cl);
+    return D == 64 ? prepare_fused_t<float, 64>(G, need, cl) : prepare_fused_t<float, 128>(G, need, cl);
 }
 
 size_t fused_attention_smem_bytes(bool bf16, int D, int G) {

@@ -26,7 +26,7 @@
 //     chunk of units, publishes one list per row, and topk_merge_kernel joins
 //     the CTAs' lists (the last CTA did that alone, with dependent loads).
 // A round of three sequences at hidden 1024, vocabulary 32000, K 4 (743 MB of
-// weights): 741 us on the ring kernel that took fp32 before, 327 us here.
+// weights): 741 us on the ring kernel that took fp32 before, 297 us here.
 #include <algorithm>
 
 #include "common.cuh"
@@ -38,6 +38,7 @@ namespace {
 constexpr int kMR = 4;                     // rows of W per item
 constexpr int kF32MaxWarps = 16;
 constexpr int kF32MaxRows = 32;            // activation rows of a pass (4 groups of 8)
+constexpr int kNormVecs = 8;               // 16-byte vectors per lane of a row normalised in registers
 constexpr int kStageBytes = kMR * 512;     // one k step of an item: 4 rows x 32 lanes x 16 bytes
 constexpr size_t kF32Smem = 216 * 1024;    // dynamic shared memory of one CTA alone on an SM
 constexpr size_t kF32SmemPair = 104 * 1024;  // of one of two
@@ -106,6 +107,20 @@ __device__ __forceinline__ int checked_token(const GemvArgs &a, int tok) {
     return 0;
 }
 
+__device__ __forceinline__ void add_squares(float4 &q, const float4 &f) {
+    q.x = fmaf(f.x, f.x, q.x);
+    q.y = fmaf(f.y, f.y, q.y);
+    q.z = fmaf(f.z, f.z, q.z);
+    q.w = fmaf(f.w, f.w, q.w);
+}
+// 1 / RMS of a row from the lanes' sums of squares.
+__device__ __forceinline__ float inv_rms(const float4 &q, const GemvArgs &a) {
+    float ss = (q.x + q.y) + (q.z + q.w);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
+    return 1.0f / sqrtf(ss / (float)a.d + a.eps);
+}
+
 // Activation rows t0 .. t0 + rows - 1 into X [rows][kin] (rows past a.T are
 // zeros).  The CTA's warps share the rows out; the warps of one row each sum
 // its squares themselves, so that no barrier separates the norm's two halves.
@@ -136,26 +151,35 @@ __device__ __forceinline__ void stage_rows(const GemvArgs &a, int t0, int rows, 
             const int sr = a.src_prefill_rows ? t * a.max_new + clamp_new(a, t) - 1 : t;
             s0 = (const float4 *)(a.src + (size_t)sr * a.d);
             g = (const float4 *)a.gain;
+            if (g && nvec <= kNormVecs * 32) {
+                // the row in registers: one round trip for the sum and the values
+                float4 f[kNormVecs];
+#pragma unroll
+                for (int i = 0; i < kNormVecs; ++i) f[i] = lane + 32 * i < nvec ? __ldcg(s0 + lane + 32 * i) : zero;
+                float4 q = zero;
+#pragma unroll
+                for (int i = 0; i < kNormVecs; ++i) add_squares(q, f[i]);
+                inv = inv_rms(q, a);
+#pragma unroll
+                for (int i = 0; i < kNormVecs; ++i) {
+                    const int v = lane + 32 * i;
+                    if (v >= nvec || i % wpr != share) continue;
+                    const float4 w = __ldg(g + v);
+                    x[v] = make_float4(f[i].x * inv * w.x, f[i].y * inv * w.y, f[i].z * inv * w.z, f[i].w * inv * w.w);
+                }
+                continue;
+            }
             if (g) {
                 float4 q = zero;
 #pragma unroll 4
-                for (int v = lane; v < nvec; v += 32) {
-                    const float4 f = __ldcg(s0 + v);
-                    q.x = fmaf(f.x, f.x, q.x);
-                    q.y = fmaf(f.y, f.y, q.y);
-                    q.z = fmaf(f.z, f.z, q.z);
-                    q.w = fmaf(f.w, f.w, q.w);
-                }
-                float ss = (q.x + q.y) + (q.z + q.w);
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xFFFFFFFFu, ss, o);
-                inv = 1.0f / sqrtf(ss / (float)a.d + a.eps);
+                for (int v = lane; v < nvec; v += 32) add_squares(q, __ldcg(s0 + v));
+                inv = inv_rms(q, a);
             }
         } else {
             s0 = (const float4 *)((const float *)a.act + (size_t)t * a.kin);
         }
         const bool pair = s1 != nullptr;
-#pragma unroll 4
+#pragma unroll 8
         for (int v = share * 32 + lane; v < nvec; v += wpr * 32) {
             float4 f = !s0 ? zero : pair && v >= dv ? __ldcg(s1 + (v - dv)) : __ldcg(s0 + v);
             if (g) {
@@ -217,6 +241,9 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
 
     const int per_chunk = TOPK ? p.chunk : max(i1 - i0, 1);
     start_copies(i0, min(i0 + per_chunk, i1));
+    // the gain is a weight: requested early, it is in L2 when the rows are normalised
+    if (a.pro == kProNorm && a.gain && threadIdx.x * 32 < a.d)
+        asm volatile("prefetch.global.L2 [%0];" ::"l"((const float *)a.gain + threadIdx.x * 32) : "memory");
     pdl_wait();
 
     for (int pass = 0; pass < n_pass; ++pass) {
@@ -372,7 +399,7 @@ bool f32_plan(const GemvArgs &a, int grid, F32Plan &p, size_t &smem) {
                     long best = -1;
                     for (int seg = 1; seg * p.tg <= p.warps && seg <= nk; seg *= 2) {
                         const int groups = p.warps / (seg * p.tg);
-                        const long cost = (long)((per_cta + groups - 1) / groups) * ((nk + seg - 1) / seg + 3);
+                        const long cost = (long)((per_cta + groups - 1) / groups) * ((nk + seg - 1) / seg + 1);
                         if (best < 0 || cost < best) { best = cost; p.seg = seg; }
                     }
                     return true;

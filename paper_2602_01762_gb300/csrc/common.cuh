@@ -232,29 +232,73 @@ __device__ __forceinline__ void key_insert(Key (&l)[kTopK], Key k) {
     }
 }
 
-// Lanes lane and lane ^ m both end with the best kTopK keys of their two
-// lists: the element-wise maximum of one list and the other reversed is that
-// set as a bitonic sequence, sorted by three half-cleaner stages.  Every lane
-// of the warp takes part.
-__device__ __forceinline__ void key_merge_xor(Key (&l)[kTopK], int m) {
-    Key c[kTopK];
+// l becomes the best kTopK keys of two sorted lists: the element-wise maximum
+// of one list and the other reversed is that set as a bitonic sequence, sorted
+// by three half-cleaner stages.
+__device__ __forceinline__ void key_merge_rev(Key (&l)[kTopK], const Key (&rev)[kTopK]) {
 #pragma unroll
-    for (int i = 0; i < kTopK; ++i) {
-        const Key o = __shfl_xor_sync(0xFFFFFFFFu, l[kTopK - 1 - i], m);
-        c[i] = l[i] > o ? l[i] : o;
-    }
+    for (int i = 0; i < kTopK; ++i) l[i] = l[i] > rev[i] ? l[i] : rev[i];
 #pragma unroll
     for (int d = kTopK / 2; d > 0; d >>= 1)
 #pragma unroll
         for (int i = 0; i < kTopK; ++i)
             if ((i & d) == 0) {
-                const Key x = c[i], y = c[i + d];
-                c[i] = x > y ? x : y;
-                c[i + d] = x > y ? y : x;
+                const Key x = l[i], y = l[i + d];
+                l[i] = x > y ? x : y;
+                l[i + d] = x > y ? y : x;
             }
-#pragma unroll
-    for (int i = 0; i < kTopK; ++i) l[i] = c[i];
 }
+
+// Lanes lane and lane ^ m both end with the best kTopK keys of their two
+// lists.  Every lane of the warp takes part.
+__device__ __forceinline__ void key_merge_xor(Key (&l)[kTopK], int m) {
+    Key o[kTopK];
+#pragma unroll
+    for (int i = 0; i < kTopK; ++i) o[i] = __shfl_xor_sync(0xFFFFFFFFu, l[kTopK - 1 - i], m);
+    key_merge_rev(l, o);
+}
+
+// The per-CTA lists of one row ([n][kTopK] values and ids, 16-byte aligned, each
+// sorted; id -1: an empty place) merged by 128 threads: thread e takes the lists
+// e, e + 128, ... whole.  load() requests the first two; join() uses them.
+struct ListShare {
+    float4 v[2][2];
+    int4 id[2][2];
+    __device__ __forceinline__ void load1(int s, const float *pv, const int *pi, int n, int c) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            v[s][h] = c < n ? __ldcg((const float4 *)(pv + (size_t)c * kTopK) + h) : make_float4(0.f, 0.f, 0.f, 0.f);
+            id[s][h] = c < n ? __ldcg((const int4 *)(pi + (size_t)c * kTopK) + h) : make_int4(-1, -1, -1, -1);
+        }
+    }
+    __device__ __forceinline__ void load(const float *pv, const int *pi, int n, int e) {
+        load1(0, pv, pi, n, e);
+        load1(1, pv, pi, n, e + 128);
+    }
+    static __device__ __forceinline__ Key key(float v, int id) { return id >= 0 ? pack_best(v, id) : 0ull; }
+    __device__ __forceinline__ void join(Key (&l)[kTopK], const float *pv, const int *pi, int n, int e) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            l[4 * h] = key(v[0][h].x, id[0][h].x);
+            l[4 * h + 1] = key(v[0][h].y, id[0][h].y);
+            l[4 * h + 2] = key(v[0][h].z, id[0][h].z);
+            l[4 * h + 3] = key(v[0][h].w, id[0][h].w);
+        }
+#pragma unroll 1
+        for (int c = e + 128; c < n; c += 128) {
+            Key r[kTopK];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                r[7 - 4 * h] = key(v[1][h].x, id[1][h].x);
+                r[6 - 4 * h] = key(v[1][h].y, id[1][h].y);
+                r[5 - 4 * h] = key(v[1][h].z, id[1][h].z);
+                r[4 - 4 * h] = key(v[1][h].w, id[1][h].w);
+            }
+            key_merge_rev(l, r);
+            load1(1, pv, pi, n, c + 128);
+        }
+    }
+};
 
 // Entry r of a register list without a dynamic index.
 __device__ __forceinline__ Key key_at(const Key (&l)[kTopK], int r) {

@@ -572,29 +572,14 @@ __global__ void __launch_bounds__(256) tree_lse_kernel(const TreeArgs a) {
         if (lane == 0) a.lse[t] = M + logf(S);
     } else if (a.lm_val && a.lm_lse_grid > 0 && warp <= 4) {
         // warps 1-4: the LM head's per-CTA top-8 lists of this row, merged
-        // (every load of a thread's share first, then its insertions, then
-        // each warp's lists across lanes)
         const int lm_row = a.step == 1 ? b : t;
-        const int nc = a.lm_lse_grid * kTopK, e = tid - 32;
+        const int nc = a.lm_lse_grid * kTopK;
+        Key l[kTopK];
         const float *pv = a.lm_val + (size_t)lm_row * nc;
         const int *pi = a.lm_id + (size_t)lm_row * nc;
-        constexpr int kB = 16;
-        float v[kB];
-        int id[kB];
-#pragma unroll
-        for (int q = 0; q < kB; ++q) {
-            const int c = e + q * 128;
-            v[q] = c < nc ? __ldcg(pv + c) : 0.f;
-            id[q] = c < nc ? __ldcg(pi + c) : -1;
-        }
-        Key l[kTopK];
-        key_clear(l);
-#pragma unroll 1
-        for (int q = 0; q < kB; ++q)
-            if (id[q] >= 0) key_insert(l, pack_best(v[q], id[q]));
-#pragma unroll 1
-        for (int c = e + kB * 128; c < nc; c += 128)
-            if (__ldcg(pi + c) >= 0) key_insert(l, pack_best(__ldcg(pv + c), __ldcg(pi + c)));
+        ListShare ls;
+        ls.load(pv, pi, a.lm_lse_grid, tid - 32);
+        ls.join(l, pv, pi, a.lm_lse_grid, tid - 32);
 #pragma unroll 1
         for (int m = 1; m < 32; m <<= 1) key_merge_xor(l, m);
         if (lane == 0)
@@ -606,9 +591,9 @@ __global__ void __launch_bounds__(256) tree_lse_kernel(const TreeArgs a) {
         // the row's top-w candidates, ranked (logit descending, then id ascending)
         Key l[kTopK];
 #pragma unroll
-        for (int i = 0; i < kTopK; ++i) l[i] = lane < 4 ? s_k[lane][i] : 0ull;
+        for (int i = 0; i < kTopK; ++i) l[i] = s_k[lane & 3][i];
 #pragma unroll 1
-        for (int m = 1; m < 32; m <<= 1) key_merge_xor(l, m);
+        for (int m = 1; m < 4; m <<= 1) key_merge_xor(l, m);
         if (lane < a.w) {
             float v;
             int id;

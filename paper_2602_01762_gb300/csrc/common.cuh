@@ -565,6 +565,9 @@ bool gemv_supported(const GemvArgs &a, bool bf16);
 // fp32 projections (gemv_f32.cu); a selection's lists are joined by the merge kernel.
 cudaError_t prepare_gemv_f32_kernels();
 cudaError_t launch_gemv_f32(const GemvArgs &a, int grid, cudaStream_t s, bool pdl);
+// Gate/up + SwiGLU of one bf16 activation row (a copy prologue) on the same kernel.
+bool gemv_pair_supported(const GemvArgs &a, int grid);
+cudaError_t launch_gemv_pair(const GemvArgs &a, int grid, cudaStream_t s, bool pdl);
 // Joins the per-CTA top-k lists ([T][slots][8] in lm_part / lm_part_id) of a selection.
 cudaError_t launch_topk_merge(const GemvArgs &a, int slots, cudaStream_t s);
 bool gemv_mma_supported(const GemvArgs &a);

@@ -25,6 +25,11 @@
 //   * The LM head keeps the CTA's logits in shared memory, selects once per
 //     chunk of units, publishes one list per row, and topk_merge_kernel joins
 //     the CTAs' lists (the last CTA did that alone, with dependent loads).
+// Gate/up + SwiGLU of one bf16 row takes the same kernel, on the row that the O
+// projection's finish kernel wrote: the ring kernel spends 44 warp instructions on
+// 512 bytes of weights, this one 16 (rounds of one sequence: 70B shape 3288 us
+// there and 3099 here, 8B shape 1283 and 1279, 7B shape 987 and 982; on the tcgen05
+// kernel the 8B shape took 1291 against 1281 on the ring kernel).
 // A round of three sequences at hidden 1024, vocabulary 32000, K 4 (743 MB of
 // weights): 741 us on the ring kernel that took fp32 before, 297 us here.
 #include <algorithm>
@@ -68,6 +73,11 @@ __device__ __forceinline__ void cp_wait(int S) {
 }
 __device__ __forceinline__ void ffma2(unsigned long long &acc, unsigned long long a, unsigned long long b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+
+// A packed bf16 pair as two floats (exact).
+__device__ __forceinline__ unsigned long long widen2(uint32_t w) {
+    return ((unsigned long long)(w & 0xFFFF0000u) << 32) | (w << 16);
 }
 
 // The sums of N values over the 32 lanes: lane l ends with the sum of value
@@ -122,9 +132,22 @@ __device__ __forceinline__ float inv_rms(const float4 &q, const GemvArgs &a) {
 }
 
 // Activation rows t0 .. t0 + rows - 1 into X [rows][kin] (rows past a.T are
-// zeros).  The CTA's warps share the rows out; the warps of one row each sum
+// zeros; bf16 rows are copied, and laid out as two planes).  The CTA's warps share the rows out; the warps of one row each sum
 // its squares themselves, so that no barrier separates the norm's two halves.
+template <typename WT>
 __device__ __forceinline__ void stage_rows(const GemvArgs &a, int t0, int rows, float *X) {
+    if constexpr (sizeof(WT) == 2) {
+        const int nv = a.kin / 8;
+        for (int e = threadIdx.x; e < rows * nv; e += blockDim.x) {
+            const int r = e / nv, v = e % nv;
+            const uint4 q = t0 + r < a.T ? __ldcg((const uint4 *)((const uint16_t *)a.act + (size_t)(t0 + r) * a.kin) + v)
+                                         : make_uint4(0u, 0u, 0u, 0u);
+            float4 *x = (float4 *)(X + (size_t)r * a.kin);
+            x[v] = make_float4(bf16lo(q.x), bf16hi(q.x), bf16lo(q.y), bf16hi(q.y));
+            x[nv + v] = make_float4(bf16lo(q.z), bf16hi(q.z), bf16lo(q.w), bf16hi(q.w));
+        }
+        return;
+    }
     const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int wpr = rows < warps ? warps / rows : 1, share = warp % wpr;
     const int nvec = a.kin / 4, dv = a.d / 4;
@@ -192,14 +215,15 @@ __device__ __forceinline__ void stage_rows(const GemvArgs &a, int t0, int rows, 
 }
 
 // TN: activation rows per warp.  RPW: rows of W per unit (2: gate and up).
-template <int TN, int RPW, bool TOPK>
-__global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const GemvArgs a, const F32Plan p) {
+template <typename WT, int TN, int RPW, bool TOPK>
+__global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_rows4_kernel(const GemvArgs a, const F32Plan p) {
     extern __shared__ __align__(16) uint8_t smem_raw[];
     __shared__ float s_part[2][kF32MaxWarps][32];                  // segments' sums, double-buffered by item
     __shared__ Key s_list[TOPK ? kF32MaxRows : 1][kTopK];          // selections of the chunks so far
     constexpr int N = kMR * TN, UI = kMR / RPW, LPV = 32 / N;      // sums, units per item, lanes per sum
+    constexpr int VEC = Elem<WT>::kPerVec;
     const int warps = blockDim.x >> 5, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int S = p.stages, seg = p.seg, rows = p.tg * TN, nvec = a.kin / 4;
+    const int S = p.stages, seg = p.seg, rows = p.tg * TN, nvec = a.kin / VEC;
     const int sg = warp % seg, tgi = warp / seg % p.tg, groups = warps / (seg * p.tg), grp = warp / (seg * p.tg);
     const int v_lo = (int)((long)sg * nvec / seg), v_hi = (int)((long)(sg + 1) * nvec / seg);
     const int nks = (v_hi - v_lo + 31) / 32;
@@ -220,7 +244,7 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
         if (ci < cend) {
             const int v = v_lo + cks * 32 + lane;
             if (v < v_hi) {
-                const float *w = (const float *)a.W + (size_t)v * 4;
+                const WT *w = (const WT *)a.W + (size_t)v * VEC;
 #pragma unroll
                 for (int r = 0; r < kMR; ++r) {
                     const int u = min(ci * UI + r % UI, a.n_units - 1) + (r / UI) * a.pair_offset;
@@ -249,7 +273,7 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
     for (int pass = 0; pass < n_pass; ++pass) {
         const int t0 = pass * rows, tc = min(rows, a.T - t0);
         if (pass) __syncthreads();
-        stage_rows(a, t0, rows, X);
+        stage_rows<WT>(a, t0, rows, X);
         __syncthreads();
         int c0 = i0;
         do {
@@ -274,11 +298,24 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
                         const ulonglong2 *x = (const ulonglong2 *)(X + (size_t)(tgi * TN) * a.kin) + v;
 #pragma unroll
                         for (int t = 0; t < TN; ++t) {
-                            const ulonglong2 xv = x[(size_t)t * nvec];
+                            if constexpr (VEC == 4) {
+                                const ulonglong2 xv = x[(size_t)t * nvec];
 #pragma unroll
-                            for (int r = 0; r < kMR; ++r) {
-                                ffma2(acc[r][t], w[r].x, xv.x);
-                                ffma2(acc[r][t], w[r].y, xv.y);
+                                for (int r = 0; r < kMR; ++r) {
+                                    ffma2(acc[r][t], w[r].x, xv.x);
+                                    ffma2(acc[r][t], w[r].y, xv.y);
+                                }
+                            } else {
+                                // eight weights, widened exactly; X holds the first and the last
+                                // four of every eight activations as two planes (no bank conflicts)
+                                const ulonglong2 xa = x[(size_t)t * 2 * nvec], xb = x[(size_t)t * 2 * nvec + nvec];
+#pragma unroll
+                                for (int r = 0; r < kMR; ++r) {
+                                    ffma2(acc[r][t], widen2((uint32_t)w[r].x), xa.x);
+                                    ffma2(acc[r][t], widen2((uint32_t)(w[r].x >> 32)), xa.y);
+                                    ffma2(acc[r][t], widen2((uint32_t)w[r].y), xb.x);
+                                    ffma2(acc[r][t], widen2((uint32_t)(w[r].y >> 32)), xb.y);
+                                }
                             }
                         }
                     }
@@ -309,7 +346,7 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
                     if (a.logits) a.logits[((size_t)t * a.K + a.step - 1) * a.vocab + u] = z;
                     Z[(size_t)tl * zs + (u - c0 * UI)] = z;
                 } else if constexpr (RPW == 2) {
-                    ((float *)a.out_act)[(size_t)t * a.out_ld + u] = z / (1.0f + expf(-z)) * up;
+                    Elem<WT>::store((WT *)a.out_act, (size_t)t * a.out_ld + u, z / (1.0f + expf(-z)) * up);
                 } else {
                     if (a.epi == kEpiResid) {
                         z += a.resid[(size_t)(a.resid_prefill_rows ? t * a.max_new + clamp_new(a, t) - 1 : t) * a.out_ld + u];
@@ -358,28 +395,34 @@ __global__ void __launch_bounds__(kF32MaxWarps * 32, 1) gemv_f32_kernel(const Ge
 template <int TN>
 cudaError_t dispatch_f32(const GemvArgs &a, const F32Plan &p, int grid, size_t smem, cudaStream_t s, bool pdl) {
     const dim3 g(grid), b(p.warps * 32);
-    if (a.epi == kEpiTopK) return launch_k(gemv_f32_kernel<TN, 1, true>, g, b, smem, s, pdl, a, p);
-    if (a.epi == kEpiSwiGLU) return launch_k(gemv_f32_kernel<TN, 2, false>, g, b, smem, s, pdl, a, p);
-    return launch_k(gemv_f32_kernel<TN, 1, false>, g, b, smem, s, pdl, a, p);
+    if (a.epi == kEpiTopK) return launch_k(gemv_rows4_kernel<float, TN, 1, true>, g, b, smem, s, pdl, a, p);
+    if (a.epi == kEpiSwiGLU) return launch_k(gemv_rows4_kernel<float, TN, 2, false>, g, b, smem, s, pdl, a, p);
+    return launch_k(gemv_rows4_kernel<float, TN, 1, false>, g, b, smem, s, pdl, a, p);
 }
 
 template <int TN>
 cudaError_t f32_attrs() {
-    cudaError_t e = cudaFuncSetAttribute(gemv_f32_kernel<TN, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
+    cudaError_t e = cudaFuncSetAttribute(gemv_rows4_kernel<float, TN, 1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gemv_f32_kernel<TN, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
+        e = cudaFuncSetAttribute(gemv_rows4_kernel<float, TN, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(gemv_f32_kernel<TN, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
+        e = cudaFuncSetAttribute(gemv_rows4_kernel<float, TN, 1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
     return e;
+}
+
+// A layer with fewer bytes per CTA than this runs as 8-warp CTAs, two to an SM.
+bool small_layer(const GemvArgs &a, int es, int grid) {
+    const int UI = a.epi == kEpiSwiGLU ? kMR / 2 : kMR;
+    const int n_items = (a.n_units + UI - 1) / UI, per_cta = (n_items + grid - 1) / grid;
+    return (size_t)per_cta * kMR * a.kin * es < 384 * 1024;
 }
 
 // The most activation rows per pass that fit beside the smallest ring, then
 // the largest ring; then the segment count with the shortest run of k steps.
-bool f32_plan(const GemvArgs &a, int grid, F32Plan &p, size_t &smem) {
+bool f32_plan(const GemvArgs &a, int es, int grid, F32Plan &p, size_t &smem) {
     const int UI = a.epi == kEpiSwiGLU ? kMR / 2 : kMR;
     const int n_items = (a.n_units + UI - 1) / UI, per_cta = (n_items + grid - 1) / grid;
-    // a CTA's weights in bytes: below this two 8-warp CTAs to an SM
-    const bool small = (size_t)per_cta * kMR * a.kin * 4 < 384 * 1024;
+    const bool small = small_layer(a, es, grid);
     // beside such CTAs the next layer's own rings are already filling: requests
     // for its first bytes only delay them (339 us a round with, 327 without, three sequences as above)
     p.prefetch = !small;
@@ -395,7 +438,7 @@ bool f32_plan(const GemvArgs &a, int grid, F32Plan &p, size_t &smem) {
             for (int S : {6, 4, 2})
                 if ((smem = (size_t)p.warps * S * kStageBytes + x) <= room) {
                     p.stages = S;
-                    const int nk = (a.kin / 4 + 31) / 32;
+                    const int nk = (a.kin * es / 16 + 31) / 32;
                     long best = -1;
                     for (int seg = 1; seg * p.tg <= p.warps && seg <= nk; seg *= 2) {
                         const int groups = p.warps / (seg * p.tg);
@@ -418,13 +461,31 @@ cudaError_t prepare_gemv_f32_kernels() {
     if (e == cudaSuccess) e = f32_attrs<2>();
     if (e == cudaSuccess) e = f32_attrs<4>();
     if (e == cudaSuccess) e = f32_attrs<8>();
+    if (e == cudaSuccess)
+        e = cudaFuncSetAttribute(gemv_rows4_kernel<uint16_t, 1, 2, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kF32Smem);
     return e;
+}
+
+bool gemv_pair_supported(const GemvArgs &a, int grid) {
+    F32Plan p{};
+    size_t smem;
+    // (a small layer stays on the ring kernel, which norms its row itself: hidden
+    // 1024, batch 1, 198 us a round there and 207 here)
+    return a.epi == kEpiSwiGLU && a.T == 1 && !small_layer(a, 2, grid) && f32_plan(a, 2, grid, p, smem);
+}
+
+cudaError_t launch_gemv_pair(const GemvArgs &a, int grid, cudaStream_t s, bool pdl) {
+    F32Plan p{};
+    size_t smem;
+    if (a.pro != kProCopy || !gemv_pair_supported(a, grid) || !f32_plan(a, 2, grid, p, smem)) return cudaErrorInvalidValue;
+    p.prefetch = 1;
+    return launch_k(gemv_rows4_kernel<uint16_t, 1, 2, false>, dim3(grid), dim3(p.warps * 32), smem, s, pdl, a, p);
 }
 
 cudaError_t launch_gemv_f32(const GemvArgs &a, int grid, cudaStream_t s, bool pdl) {
     F32Plan p{};
     size_t smem;
-    if (!f32_plan(a, grid, p, smem)) return cudaErrorInvalidValue;
+    if (!f32_plan(a, 4, grid, p, smem)) return cudaErrorInvalidValue;
     cudaError_t e = p.tn == 1   ? dispatch_f32<1>(a, p, grid, smem, s, pdl)
                     : p.tn == 2 ? dispatch_f32<2>(a, p, grid, smem, s, pdl)
                     : p.tn == 4 ? dispatch_f32<4>(a, p, grid, smem, s, pdl)

@@ -286,6 +286,11 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
     auto on_tc_staged = [&](const GemvArgs &g, const CUtensorMap *tm) -> bool {
         return tm && want_tc(g) && c->tc_ready && c->bf16 && gemv_tc_supported(g, c->sms);
     };
+    // gate/up of one row whose bf16 row the O projection's finish kernel wrote
+    auto on_pair = [&](const GemvArgs &g, const CUtensorMap *tm) -> bool {
+        return tm && c->gemv_tcgen05 == 1 && c->tc_ready && c->bf16 && c->tc_stream_rows <= 1 &&
+               gemv_pair_supported(g, gemv_grid(c, g.n_units));
+    };
     // x_ready: the bf16 buffer already holds the rows of the next projection,
     // written by the previous projection's last kernel
     bool x_ready = false;
@@ -297,7 +302,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
                 g.act = c->xbuf;
             }
             x_ready = false;
-            if (c->fuse_rows && next && next->T == g.T && on_tcs(*next, ntm)) {
+            if (c->fuse_rows && next && next->T == g.T && (on_tcs(*next, ntm) || on_pair(*next, ntm))) {
                 if (g.epi == kEpiTopK && next->pro == kProFuseDecode) {
                     g.next_fuse = 1;
                     g.next_x = c->xbuf;
@@ -312,6 +317,12 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             const cudaError_t le = launch_gemv_tcs(g, *tm, c->sms, c->tc_part, c->tc_ctr, c->xbuf, s, pdl_here, &done);
             x_ready = le == cudaSuccess && done;
             return le;
+        }
+        if (x_ready && on_pair(g, tm)) {
+            x_ready = false;
+            g.pro = kProCopy;
+            g.act = c->xbuf;
+            return launch_gemv_pair(g, grid, s, pdl_here);
         }
         x_ready = false;
         if (on_tc_staged(g, tm)) {

@@ -419,7 +419,8 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * SM), "prefetch_next_kb" (16384, the default: once a kernel's CTAs have
  * requested their last weight boxes, they request the first this many KB of
  * the next kernel's weights into L2, each CTA an even share, so that HBM
- * keeps streaming across the kernel boundary; 0: none),
+ * keeps streaming across the kernel boundary; none of a layer that fits the
+ * rings of one CTA per SM; 0: none),
  * "fuse_rows" (1, the default: a streamed projection's last kernel, the
  * split-K finish or the LM head's top-k merge, also writes the next
  * projection's bf16 activation rows, its RMSNorm or the next step's fusion

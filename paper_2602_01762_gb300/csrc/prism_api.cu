@@ -16,6 +16,7 @@ using namespace prism;
 namespace {
 
 constexpr int kGraphCache = 8;
+constexpr size_t kRingBytes = 200 * 1024;   // weights that one projection CTA's ring holds
 constexpr int kAttnLongCtx = 3072;   // cache rows beyond which two-CTA attention clusters keep 8 warps
 constexpr int kMaxProfileKernels = 12 * kMaxSteps + 8;
 
@@ -564,11 +565,13 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
     };
     const CUtensorMap *lm_tm = c->tm_lm_ok ? &c->tm_lm : nullptr;
     // a kernel's CTAs, once their own weights are requested, request the next
-    // kernel's first bytes into L2
+    // kernel's first bytes into L2, unless the rings of the next kernel's early
+    // CTAs take all of them anyway (hidden 1024, batch 1 199.5 us a round with the
+    // requests, 197 without; batch 20 279 and 276; nothing changes at hidden 4096)
     const size_t wes = c->bf16 ? 2 : 4;
     auto pf = [&](const void *w, size_t elems) -> std::pair<const void *, long long> {
         const long long cap = (long long)c->prefetch_next_kb * 1024;
-        if (!w || cap <= 0) return {nullptr, 0};
+        if (!w || cap <= 0 || elems * wes <= (size_t)c->sms * kRingBytes) return {nullptr, 0};
         return {w, std::min(cap, (long long)(elems * wes))};
     };
     auto with_pf = [&](GemvArgs g, std::pair<const void *, long long> n) {

@@ -369,9 +369,8 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * per tile adds the sums itself; a greedy LM head other than that streamed
  * top-1 below (lm_stream) streams from max(this, 8) rows outside tree rounds), "attn_ctas_per_sm" (1..64, default 2: the fused attention
  * kernel's cluster size halves while batch x KV heads x cluster size exceeds
- * this many CTAs per SM, while half as many CTAs already take the whole cache
- * (max_ctx) in one stage each, and, above 2, while the device cannot hold all
- * clusters of that size at once), "gemv_cuda_core" (for projections
+ * this many CTAs per SM and, above 2 and with caches of 8 MB or more, while
+ * the device cannot hold all clusters of that size at once), "gemv_cuda_core" (for projections
  * not on the tcgen05 kernel, bf16: 1, the default, the CUDA-core TMA-ring
  * kernel; 0: the warp-level mma.sync kernel), "attn_fused" (1, the default: RoPE,
  * KV append and attention run as one kernel, a cluster of up to 8 CTAs per
@@ -384,7 +383,8 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
  * kernel: 8, stages of 128 keys, one CTA per SM; or 4, stages of 64 keys,
  * two CTAs per SM; 0, the default: 4 where the CTAs are more than the SMs,
  * except clusters of two over caches of more than 3072 rows and several
- * sequences, else 8), "attn_lpt" (1,
+ * sequences, and caches below 8 MB unless one CTA per (sequence, KV head)
+ * makes at most two per SM, else 8), "attn_lpt" (1,
  * the default: where that kernel's CTAs make more than one wave but at most
  * two, the CTAs take the sequences in order of decreasing context length;
  * 0: in index order),

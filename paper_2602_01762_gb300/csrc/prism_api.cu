@@ -17,6 +17,7 @@ namespace {
 
 constexpr int kGraphCache = 8;
 constexpr size_t kRingBytes = 200 * 1024;   // weights that one projection CTA's ring holds
+constexpr long long kAttnSmallCache = 8LL << 20;  // bytes of K and V below which attention clusters keep their size
 constexpr int kAttnLongCtx = 3072;   // cache rows beyond which two-CTA attention clusters keep 8 warps
 constexpr int kMaxProfileKernels = 12 * kMaxSteps + 8;
 
@@ -345,24 +346,23 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
     const bool tree_cluster = maps && r.tree_w > 0 && r.tree_w * (Hq / Hkv) <= kTreeClusterPairs;
 
     // CTAs per (sequence, KV head) of the attention kernels: halved while they
-    // exceed attn_ctas_per_sm per SM; while half as many already take the whole
-    // cache in one stage each, since a cluster's merge then costs more than its
-    // CTAs save (tiny drafter, batch 8, contexts 64 to 200: 177 us a round in
-    // clusters of 8, 147 so; hidden 1024, batch 6, contexts to 400: 335 and 306);
-    // and while the device cannot hold all clusters at once: the second wave of
-    // clusters of 4 or 8 starts only when that many SMs of one GPC are free, and
-    // costs a whole launch's latency again (8B shape, batch 4, contexts to 4096, clusters
-    // of 8 and of 4: 1405 us a round and 1325; the 7B shape at batch 1 1069 and 980; the
-    // tree of 4 sequences 1192 and 1116).  pair_fits: clusters of two may take two waves
-    auto attn_cluster = [&](int most, int stage_keys, bool pair_fits) {
+    // exceed attn_ctas_per_sm per SM, and while the device cannot hold all
+    // clusters at once: the second wave of clusters of 4 or 8 starts only when
+    // that many SMs of one GPC are free, and costs a whole launch's latency again
+    // (8B shape, batch 4, contexts to 4096, clusters of 8 and of 4: 1405 us a round
+    // and 1325; the 7B shape at batch 1 1069 and 980; the tree of 4 sequences 1192
+    // and 1116).  pair_fits: clusters of two may take two waves.  Small caches keep
+    // their clusters: the order of their sums decides nearly tied candidates of
+    // small drafters (tiny drafter, batch 8, contexts to 200: 147 us, 177 so)
+    const bool small_cache = (long long)r.B * Hkv * f.max_ctx * D * 2 * (c->bf16 ? 2 : 4) < kAttnSmallCache;
+    auto attn_cluster = [&](int most, bool pair_fits) {
         const long long pairs = (long long)r.B * Hkv;
         auto fits = [&](int cs) {
             const int n = cs > 8 ? 0 : c->attn_cl.resident[cs == 8 ? 2 : cs == 4 ? 1 : 0];
-            return (cs == 2 && pair_fits) || n == 0 || pairs <= n;
+            return small_cache || (cs == 2 && pair_fits) || n == 0 || pairs <= n;
         };
         int cs = most;
-        while (cs > 1 && (pairs * cs > (long long)c->attn_ctas_per_sm * c->sms || (long long)(cs / 2) * stage_keys >= f.max_ctx ||
-                          !fits(cs))) cs /= 2;
+        while (cs > 1 && (pairs * cs > (long long)c->attn_ctas_per_sm * c->sms || !fits(cs))) cs /= 2;
         return cs;
     };
 
@@ -613,7 +613,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             const auto n = pf(c->steps[k - 1].w_o, (size_t)d * Hq * D);
             ta.pf_next = n.first;
             ta.pf_next_bytes = n.second;
-            e = tree_cluster ? launch_tree_cluster_attention(ta, attn_cluster(std::min(c->attn_cl.most, 8), 128, false), tmk, tmv, s, pdl)
+            e = tree_cluster ? launch_tree_cluster_attention(ta, attn_cluster(std::min(c->attn_cl.most, 8), false), tmk, tmv, s, pdl)
                              : launch_tree_attention(ta, c->bf16, s, pdl);
             after(3);
             if (e != cudaSuccess) break;
@@ -636,7 +636,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             fa.Hkv = Hkv;
             fa.D = D;
             fa.max_ctx = f.max_ctx;
-            fa.cs = attn_cluster(c->attn_cl.most, c->bf16 ? 128 : 32, true);
+            fa.cs = attn_cluster(c->attn_cl.most, true);
             fa.err = c->err;
             fa.wait_polls = c->wait_polls;
             {
@@ -650,10 +650,12 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             // and 1875).  Clusters of two in two waves over long caches keep 8 warps:
             // twice the bytes in flight per CTA and, with the longest sequences first,
             // a short tail (8B shape, contexts 512 to 4096, batch 12: 1430 us with 8,
-            // 1472 with 4; contexts 512 to 2000: 1413 and 1406)
+            // 1472 with 4; contexts 512 to 2000: 1413 and 1406).  Small caches: one wave
+            // of single CTAs only (as for their clusters)
             const long long n_ctas = (long long)r.B * Hkv * fa.cs;
             const bool long_pairs = fa.cs == 2 && r.B > 1 && f.max_ctx > kAttnLongCtx;
-            fa.warps = c->attn_warps ? c->attn_warps : n_ctas > c->sms && !long_pairs ? 4 : 8;
+            const bool four = small_cache ? fa.cs == 1 && n_ctas <= 2LL * c->sms : !long_pairs;
+            fa.warps = c->attn_warps ? c->attn_warps : n_ctas > c->sms && four ? 4 : 8;
             if (fa.warps == 4 && fa.cs > 8) fa.cs = 8;   // clusters of 16 are checked for the 8-warp kernel only
             // more than one wave of CTAs but at most two: the longest sequences
             // first (with more waves the hardware's scheduling already evens

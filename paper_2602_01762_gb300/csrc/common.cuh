@@ -198,6 +198,13 @@ __device__ __forceinline__ void unpack_best(unsigned long long key, float &v, in
     v = __uint_as_float((k & 0x80000000u) ? (k & 0x7FFFFFFFu) : ~k);
     id = (int)(0xFFFFFFFFu - (uint32_t)key);
 }
+// A key as a place of a selection's result: the key 0 is a place for which there
+// was no candidate (NaN logits are none), written as the id lists' own empty entry.
+__device__ __forceinline__ void unpack_place(unsigned long long key, float &v, int &id) {
+    if (key) return unpack_best(key, v, id);
+    v = -INFINITY;
+    id = 0x7FFFFFFF;
+}
 
 // Random numbers of sampled rounds: output n of SplitMix64 from state `seed`,
 // and the uniform of (stream, b, k, i) in (0, 1) (prism.h).

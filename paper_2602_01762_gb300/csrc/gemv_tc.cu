@@ -553,7 +553,7 @@ __device__ __forceinline__ void write_row(const GemvArgs &a, int t, const Key (&
     if (lane < a.topk) {
         float v;
         int id;
-        unpack_best(key_at(l, lane), v, id);
+        unpack_place(key_at(l, lane), v, id);
         const size_t o = (size_t)t * a.K + a.step - 1;
         if (lane == 0 && draft) a.draft_out[o] = id;
         if (a.topk_ids) a.topk_ids[o * a.topk + lane] = id;
@@ -618,7 +618,7 @@ __device__ __forceinline__ void top1_join(const GemvArgs &a, int T, float (&s_v)
             const Key key = atomicExch(a.best + lane, 0ull);
             float v;
             int id;
-            unpack_best(key, v, id);
+            unpack_place(key, v, id);
             const size_t o = (size_t)lane * a.K + a.step - 1;
             a.draft_out[o] = id;
             if (a.topk_ids) a.topk_ids[o] = id;
@@ -1364,7 +1364,7 @@ __global__ void __launch_bounds__(128) topk_merge_kernel(const GemvArgs a, int g
         if (lane == 0 && !smp) {
             float v;
             int id;
-            unpack_best(l[0], v, id);
+            unpack_place(l[0], v, id);
             s_tok = id;
         }
     } else if (w == 1 && smp) {

@@ -597,7 +597,7 @@ __global__ void __launch_bounds__(256) tree_lse_kernel(const TreeArgs a) {
         if (lane < a.w) {
             float v;
             int id;
-            unpack_best(key_at(l, lane), v, id);
+            unpack_place(key_at(l, lane), v, id);
             a.top_ids[(size_t)t * a.w + lane] = id;
             a.top_vals[(size_t)t * a.w + lane] = v;
         }

@@ -36,3 +36,32 @@ def test_static_head_routes(rows, hidden, vocab, topk, norm):
         own = torch.sort(logits, dim=1, descending=True, stable=True)
         assert torch.equal(ids.long(), own.indices[:, :topk]) and torch.equal(top, own.values[:, :topk])
         assert torch.equal(draft.long(), own.indices[:, 0])
+
+
+@pytest.mark.parametrize("dtype", ["bf16", "f32"])
+@pytest.mark.parametrize("rows,hidden,topk", [(1, 256, 1), (16, 256, 1), (17, 256, 1), (3, 256, 8), (64, 256, 5), (41, 8192, 8)])
+def test_places_without_a_candidate(dtype, rows, hidden, topk):
+    """NaN logits are no candidates, and a place left over holds id 0x7FFFFFFF and logit -inf, whatever the type and
+    the route: the packed top-1, lists in one pass and in several.  Here three tokens of nine have a number, of which
+    one is -inf in the odd rows; in the last row none has."""
+    import torch
+    from paper_2602_01762_gb300 import lm_head_topk_static
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    lm = torch.full((9, hidden), float("nan"), device="cuda", dtype=dt)
+    lm[2], lm[5], lm[8] = 0.5, 0.25, 0.0
+    lm[8, 1] = float("-inf")
+    h = torch.ones(rows, hidden, device="cuda")
+    h[::2, 1] = 0.0                          # -inf * 0: NaN
+    h[-1] = float("nan")
+    i32 = dict(dtype=torch.int32, device="cuda")
+    draft, ids, flags = torch.full((rows,), -7, **i32), torch.full((rows, topk), -7, **i32), torch.full((1,), -7, **i32)
+    top = torch.zeros(rows, topk, device="cuda")
+    lm_head_topk_static(h, None, lm, draft, ids, top, None, flags)
+    assert int(flags) == 0
+    none, inf = 0x7FFFFFFF, float("inf")
+    for r in range(rows):
+        n = sum(h[r].tolist()) if r < rows - 1 else 0
+        found = [] if r == rows - 1 else [(2, 0.5 * n), (5, 0.25 * n)] + ([(8, -inf)] if r % 2 else [])
+        want = (found + [(none, -inf)] * topk)[:topk]
+        assert ids[r].tolist() == [i for i, _ in want] and top[r].tolist() == [v for _, v in want], r
+        assert int(draft[r]) == want[0][0]

@@ -403,6 +403,12 @@ struct SelectSmem {
     int pos[kTreeMaxPool];
 };
 
+// A score as the orders see it: NaN counts as -inf, so that every candidate has
+// a rank of its own (were NaN neither above nor below any other, all NaN
+// candidates would rank first, more than n_nodes of them be listed and the tree's
+// outputs written past their end).
+__device__ __forceinline__ float rankable(float score) { return fmaxf(score, -INFINITY); }
+
 // Run by all kSelectThreads threads of one CTA for sequence b, once every row
 // of b has its log-sum-exp (read through L2: other CTAs wrote them).
 __device__ void select_sequence(const TreeArgs &a, int b, SelectSmem &sm) {
@@ -424,7 +430,7 @@ __device__ void select_sequence(const TreeArgs &a, int b, SelectSmem &sm) {
         const int j = tid / w, r = tid % w, t = b * w + j;
         tok = a.top_ids[(size_t)t * w + r];
         sc = s_fscore[j] + (a.top_vals[(size_t)t * w + r] - __ldcg(a.lse + t));
-        s_cs[tid] = sc;
+        s_cs[tid] = rankable(sc);
         const size_t e = (size_t)b * a.P + base + tid;
         a.pool_tok[e] = tok;
         a.pool_par[e] = s_fpool[j];
@@ -433,7 +439,8 @@ __device__ void select_sequence(const TreeArgs &a, int b, SelectSmem &sm) {
     __syncthreads();
     if (tid < nc) {
         int rank = 0;
-        for (int c = 0; c < nc; ++c) rank += (s_cs[c] > sc) || (s_cs[c] == sc && c < tid);
+        const float own = rankable(sc);
+        for (int c = 0; c < nc; ++c) rank += (s_cs[c] > own) || (s_cs[c] == own && c < tid);
         if (rank < w) {
             const int j = tid / w, o = b * w + rank;
             a.front_tok[o] = tok;
@@ -454,10 +461,10 @@ __device__ void select_sequence(const TreeArgs &a, int b, SelectSmem &sm) {
     for (int e = tid; e < P; e += kSelectThreads) s_ps[e] = __ldcg(a.pool_score + pb + e);
     __syncthreads();
     for (int e = tid; e < P; e += kSelectThreads) {
-        const float se = s_ps[e];
+        const float se = rankable(s_ps[e]);
         int rank = 0;
         for (int c = 0; c < P; ++c) {
-            const float x = s_ps[c];
+            const float x = rankable(s_ps[c]);
             rank += (x > se) || (x == se && c < e);
         }
         s_sel[e] = rank < a.n_nodes;

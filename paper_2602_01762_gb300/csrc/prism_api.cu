@@ -846,23 +846,22 @@ prism_status prism_create(const prism_config *cfg, int32_t device, prism_ctx **o
         const int kins[] = {2 * d, d, Hq * D, d, F};
         const int epis[] = {kEpiStore, kEpiStore, kEpiResid, kEpiSwiGLU, kEpiResid};
         const int pros[] = {kProFuseDecode, kProNorm, kProCopy, kProNorm, kProCopy};
-        // any batch up to max_batch may be called, and the split of more rows than
-        // one row tile holds does not grow with their number: every row count of
-        // step 1, of later steps and of tree steps is looked at
+        // any batch up to max_batch may be called, with any tree width up to
+        // max_tree_width, and the split of more rows than one row tile holds does
+        // not grow with their number: every row count of a round is looked at
+        // (`per` rows a sequence; 0: the max_new of step 1)
         for (int i = 0; i < 5; ++i)
             for (int nb = 1; nb <= f.max_batch; ++nb)
-                for (long T : {(long)nb * f.max_new, (long)nb, (long)nb * (long)TW}) {
+                for (int per = 0; per <= (int)TW; ++per) {
                     GemvArgs g{};
                     g.n_units = units[i];
                     g.kin = kins[i];
                     g.epi = epis[i];
                     g.pro = pros[i];
-                    g.T = (int)T;
-                    size_t need = gemv_tc_workspace_floats(g, c->sms);
-                    if (need > tc_floats) tc_floats = need;
-                    need = gemv_tcs_workspace_floats(g, c->sms);
-                    if (need > tc_floats) tc_floats = need;
-                    if (gemv_tc_tiles(g) > tc_tiles) tc_tiles = gemv_tc_tiles(g);
+                    g.T = nb * (per ? per : f.max_new);
+                    tc_floats = std::max({tc_floats, gemv_tc_workspace_floats(g, c->sms),
+                                          gemv_tcs_workspace_floats(g, c->sms)});
+                    tc_tiles = std::max(tc_tiles, gemv_tc_tiles(g));
                 }
     }
     size_t sizes[] = {

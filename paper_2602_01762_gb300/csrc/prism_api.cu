@@ -849,10 +849,11 @@ prism_status prism_create(const prism_config *cfg, int32_t device, prism_ctx **o
         // any batch up to max_batch may be called, with any tree width up to
         // max_tree_width, and the split of more rows than one row tile holds does
         // not grow with their number: every row count of a round is looked at
-        // (`per` rows a sequence; 0: the max_new of step 1)
+        // (`per` rows a sequence; 0: the max_new of step 1, of which only the last
+        // goes on to the O projection and the MLP)
         for (int i = 0; i < 5; ++i)
             for (int nb = 1; nb <= f.max_batch; ++nb)
-                for (int per = 0; per <= (int)TW; ++per) {
+                for (int per = i < 2 ? 0 : 1; per <= (int)TW; ++per) {
                     GemvArgs g{};
                     g.n_units = units[i];
                     g.kin = kins[i];

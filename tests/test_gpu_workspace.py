@@ -46,3 +46,24 @@ def test_a_narrower_tree_runs_as_on_a_context_of_its_own_width(batch, width):
         model.close()
     assert got[0][0] == got[1][0]
     assert all(torch.equal(a, b) for a, b in zip(got[0][1:], got[1][1:]))
+
+
+def test_a_prompts_rows_take_no_room_in_the_mlp():
+    """Only the fusion and QKV multiply every row of step 1.  At 64 sequences of the Llama-3-8B shape with 6 tokens each
+    the largest split is QKV's, three slices of 384 rows; gate/up, which runs on 64 rows, would need 84 MB for 384."""
+    import torch
+    from paper_2602_01762_gb300 import Drafter
+    s = synth.workloads.L3_8B
+    qkv = (s.n_q_heads + 2 * s.n_kv_heads) * s.head_dim
+
+    def taken(max_new):
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        dr = Drafter.from_shape(s, max_batch=64, max_ctx=128, max_new=max_new, topk=1)
+        used = before - torch.cuda.mem_get_info()[0]
+        dr.close()
+        return used
+    taken(1)                                                    # loads the kernels
+    own = 5 * 64 * (s.hidden * 4 + qkv * 4 + 2 * s.hidden * 2)  # x0, QKV and the bf16 fusion rows of 5 tokens more
+    slices = 3 * 384 * qkv * 4
+    assert taken(6) - taken(1) <= own + slices + (4 << 20)      # and the allocator's 2 MB steps

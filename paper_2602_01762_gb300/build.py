@@ -34,7 +34,7 @@ def sources() -> list[str]:
 
 def _deps() -> list[str]:
     inc = os.path.join(ROOT, "include")
-    return sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")] + \
+    return sources() + [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))] + \
         [os.path.join(inc, f) for f in os.listdir(inc)]
 
 

@@ -1569,8 +1569,8 @@ template <typename Kern>
 void cluster_limits(Kern k, size_t smem, int threads, int need, AttnClusters *c) {
     const bool wide = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
     if (!wide) cudaGetLastError();
-    c->most = wide && clusters_resident(k, smem, threads, 16) >= need ? 16 : 8;
-    for (int i = 0; i < 3; ++i) c->resident[i] = clusters_resident(k, smem, threads, 2 << i);
+    for (int i = 0; i < 4; ++i) c->resident[i] = i < 3 || wide ? clusters_resident(k, smem, threads, 2 << i) : 0;
+    c->most = c->resident[3] >= need ? 16 : 8;
 }
 
 template <typename WT, int D>

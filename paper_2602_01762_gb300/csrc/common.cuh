@@ -6,6 +6,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "attn_plan.h"
+
 namespace prism {
 
 constexpr int kMaxSteps = 16;
@@ -604,13 +606,7 @@ size_t gemv_tcs_workspace_floats(const GemvArgs &a, int sms);
 cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, float *part, int *tile_ctr,
                             uint16_t *xbuf, cudaStream_t s, bool pdl, bool *next_done = nullptr);
 cudaError_t prepare_attention_kernel(bool bf16, int D, int chunk, int G, int splits);
-// Cluster sizes of the fused attention on this device: the largest (16 only where
-// `need` such clusters can be resident at once, else 8), and how many clusters of
-// 2, 4 and 8 CTAs can be resident at once (0: unknown).
-struct AttnClusters {
-    int most, resident[3];
-};
-// Sets kernel attributes and fills *cl.
+// Sets kernel attributes and fills *cl; `need`: the KV heads of one sequence.
 cudaError_t prepare_fused_attention(bool bf16, int D, int G, int need, AttnClusters *cl);
 size_t fused_attention_smem_bytes(bool bf16, int D, int G);
 // K or V cache [heads, max_ctx, D] bf16 as a TMA tensor map of

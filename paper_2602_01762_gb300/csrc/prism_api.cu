@@ -17,8 +17,6 @@ namespace {
 
 constexpr int kGraphCache = 8;
 constexpr size_t kRingBytes = 200 * 1024;   // weights that one projection CTA's ring holds
-constexpr long long kAttnSmallCache = 8LL << 20;  // bytes of K and V below which attention clusters keep their size
-constexpr int kAttnLongCtx = 3072;   // cache rows beyond which two-CTA attention clusters keep 8 warps
 constexpr int kMaxProfileKernels = 12 * kMaxSteps + 8;
 
 struct RoundArgs {
@@ -139,7 +137,7 @@ struct prism_ctx {
     int attn_fused = 1;                                   // 1: fused RoPE/append/attention cluster kernel
     int attn_ctas_per_sm = 2;                             // fused attention: clusters shrink until B*Hkv*cs <= this * SMs
     int tc_stream_rows = 1;                               // tcgen05 projections with this many rows or more stream X
-    AttnClusters attn_cl{8, {0, 0, 0}};                   // cluster sizes the device co-schedules
+    AttnClusters attn_cl{8, {0, 0, 0, 0}};                // cluster sizes the device co-schedules
     int fuse_rows = 1;                                    // streamed projections write the next one's activation rows
     int wait_polls = 0;                                   // role-to-role wait bound (0: built in, < 0: none)
     int w_evict_first = 1;                                // weight streams with an L2 evict-first policy
@@ -345,26 +343,8 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
     const bool cache_maps = chain_maps && maps;
     const bool tree_cluster = maps && r.tree_w > 0 && r.tree_w * (Hq / Hkv) <= kTreeClusterPairs;
 
-    // CTAs per (sequence, KV head) of the attention kernels: halved while they
-    // exceed attn_ctas_per_sm per SM, and while the device cannot hold all
-    // clusters at once: the second wave of clusters of 4 or 8 starts only when
-    // that many SMs of one GPC are free, and costs a whole launch's latency again
-    // (8B shape, batch 4, contexts to 4096, clusters of 8 and of 4: 1405 us a round
-    // and 1325; the 7B shape at batch 1 1069 and 980; the tree of 4 sequences 1192
-    // and 1116).  pair_fits: clusters of two may take two waves.  Small caches keep
-    // their clusters: the order of their sums decides nearly tied candidates of
-    // small drafters (tiny drafter, batch 8, contexts to 200: 147 us, 177 so)
-    const bool small_cache = (long long)r.B * Hkv * f.max_ctx * D * 2 * (c->bf16 ? 2 : 4) < kAttnSmallCache;
-    auto attn_cluster = [&](int most, bool pair_fits) {
-        const long long pairs = (long long)r.B * Hkv;
-        auto fits = [&](int cs) {
-            const int n = cs > 8 ? 0 : c->attn_cl.resident[cs == 8 ? 2 : cs == 4 ? 1 : 0];
-            return small_cache || (cs == 2 && pair_fits) || n == 0 || pairs <= n;
-        };
-        int cs = most;
-        while (cs > 1 && (pairs * cs > (long long)c->attn_ctas_per_sm * c->sms || !fits(cs))) cs /= 2;
-        return cs;
-    };
+    const AttnSizes attn{c->sms, c->attn_ctas_per_sm, r.B, Hkv, f.max_ctx,
+                         (long long)r.B * Hkv * f.max_ctx * D * 2 * (c->bf16 ? 2 : 4)};
 
     // tree drafting: w rows per sequence from step 2 on
     const bool tree = r.tree_w > 0;
@@ -613,7 +593,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             const auto n = pf(c->steps[k - 1].w_o, (size_t)d * Hq * D);
             ta.pf_next = n.first;
             ta.pf_next_bytes = n.second;
-            e = tree_cluster ? launch_tree_cluster_attention(ta, attn_cluster(std::min(c->attn_cl.most, 8), false), tmk, tmv, s, pdl)
+            e = tree_cluster ? launch_tree_cluster_attention(ta, attn_cluster(c->attn_cl, attn, std::min(c->attn_cl.most, 8), false), tmk, tmv, s, pdl)
                              : launch_tree_attention(ta, c->bf16, s, pdl);
             after(3);
             if (e != cudaSuccess) break;
@@ -636,7 +616,10 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
             fa.Hkv = Hkv;
             fa.D = D;
             fa.max_ctx = f.max_ctx;
-            fa.cs = attn_cluster(c->attn_cl.most, true);
+            const AttnPlan ap = attn_plan(c->attn_cl, attn, c->attn_warps, c->attn_lpt);
+            fa.cs = ap.cs;
+            fa.warps = ap.warps;
+            fa.lpt = ap.lpt;
             fa.err = c->err;
             fa.wait_polls = c->wait_polls;
             {
@@ -644,26 +627,6 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
                 fa.pf_next = n.first;
                 fa.pf_next_bytes = n.second;
             }
-            // more CTAs than SMs: 4-warp CTAs, two per SM, so that one streams while
-            // the other starts or merges (8B shape, top-8, contexts 512 to 4096, batch
-            // 64: 2050 us a round with 8 warps, 2009 with 4; 7B shape, batch 16, 1937
-            // and 1875).  Clusters of two in two waves over long caches keep 8 warps:
-            // twice the bytes in flight per CTA and, with the longest sequences first,
-            // a short tail (8B shape, contexts 512 to 4096, batch 12: 1430 us with 8,
-            // 1472 with 4; contexts 512 to 2000: 1413 and 1406).  Small caches: one wave
-            // of single CTAs only (as for their clusters)
-            const long long n_ctas = (long long)r.B * Hkv * fa.cs;
-            const bool long_pairs = fa.cs == 2 && r.B > 1 && f.max_ctx > kAttnLongCtx;
-            const bool four = small_cache ? fa.cs == 1 && n_ctas <= 2LL * c->sms : !long_pairs;
-            fa.warps = c->attn_warps ? c->attn_warps : n_ctas > c->sms && four ? 4 : 8;
-            if (fa.warps == 4 && fa.cs > 8) fa.cs = 8;   // clusters of 16 are checked for the 8-warp kernel only
-            // more than one wave of CTAs but at most two: the longest sequences
-            // first (with more waves the hardware's scheduling already evens
-            // them out and each CTA's ranking of the sequences costs more than
-            // the order gains; 8B shape, batch 64, contexts 512 to 4096: 2009 us
-            // with the order, 2090 without; batch 24, one wave: 1644 and 1630)
-            const long long per_wave = (long long)c->sms * (fa.warps == 4 ? 2 : 1);
-            fa.lpt = c->attn_lpt && r.B > 1 && r.B <= 256 && n_ctas > per_wave && n_ctas <= 2 * per_wave;
             e = launch_fused_attention(fa, c->bf16, s, pdl, cache_maps ? &tmk : nullptr, cache_maps ? &tmv : nullptr);
             after(3);
             if (e != cudaSuccess) break;

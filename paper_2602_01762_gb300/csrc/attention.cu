@@ -700,6 +700,17 @@ __device__ __forceinline__ void split2(float x, float y, uint32_t &hi, uint32_t 
     hi = (uint32_t)hx | ((uint32_t)hy << 16);
     lo = (uint32_t)f32_to_bf16(x - bf16_to_f32(hx)) | ((uint32_t)f32_to_bf16(y - bf16_to_f32(hy)) << 16);
 }
+// Two floats as N bf16 parts each (what the parts before left over), packed.
+template <int N>
+__device__ __forceinline__ void split_n(float x, float y, uint32_t (&p)[N]) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+        const uint16_t hx = f32_to_bf16(x), hy = f32_to_bf16(y);
+        p[i] = (uint32_t)hx | ((uint32_t)hy << 16);
+        x -= bf16_to_f32(hx);
+        y -= bf16_to_f32(hy);
+    }
+}
 // Whole-warp bounded wait on an mbarrier phase: lane 0 polls, every lane then
 // observes the completed phase itself.  Warp-uniform result.
 __device__ __forceinline__ bool ta_wait_warp(uint64_t *bar, uint32_t parity, long limit) {
@@ -1112,15 +1123,24 @@ __global__ void __launch_bounds__(TaCfg<W>::kThreads, TaCfg<W>::kMinBlocks)
 // KV head) takes all NQ = w * G row-head pairs over one pass of the keys.  The
 // key loop is the chain kernel's above (TMA ring, keys in M, per-warp online
 // softmax, merge through distributed shared memory) with the pairs in N as NTN
-// n8 tiles (pairs past NQ are zero queries), the queries' hi and lo parts in
+// n8 tiles (pairs past NQ are zero queries), the queries' bf16 parts in
 // shared memory instead of registers, and a key at or past `base` visible to a
 // pair only where its row's ancestor mask says so.
+// More than 16 pairs ran on the CUDA cores before, in fp32: their queries and
+// probabilities are three bf16 parts, which hold all 24 bits, and their key loop takes
+// two tiles of pairs at a time, so that the parts of no more are live at once (8B
+// shape, 5 steps, context 2048, batch 4, us a round at 5 / 8 branches: CUDA cores
+// 1735 / 1918, two parts 1432 / 1527, three parts of two tiles 1443 / 1539, of one tile 1444 /
+// 1540, of all tiles 1446 / 1541).
+// Scores that cancel (terms of 2^19 that sum to 0): relative error of the step's logits
+// 0.011 at most on the CUDA cores, 0.002 with three parts, 0.8 with two.
 // The kernel this replaces gave 128 keys to a CTA, wrote every CTA's sums to
 // memory and had the last CTA of a (sequence, head) read them back: at 17
 // splits that tail was most of the launch (24 us at batch 1 and context 2048, 43
 // at 4 sequences, for 2 and 3 us of bytes).  Tree rounds of 4 branches: batch 1,
 // 6 steps, context 2048: 1705 us before, 1647 now; 4 sequences, 4 steps, context
 // 512 to 2048: 1226 and 1191.
+template <int NTN> constexpr int kTreeParts = NTN > 2 ? 3 : 2;   // bf16 parts of a query element or probability
 template <int D, int NTN>
 __global__ void __launch_bounds__(TaCfg<8>::kThreads, 1)
     tree_attention_cluster_kernel(const TreeArgs a, const __grid_constant__ CUtensorMap tk,
@@ -1128,13 +1148,14 @@ __global__ void __launch_bounds__(TaCfg<8>::kThreads, 1)
     constexpr int W = 8, kC = TaCfg<W>::kC, kThr = TaCfg<W>::kThreads, NH = D / 64, NT = D / 16, NP = 8 * NTN;
     constexpr uint32_t kBox = kC * 128, kStage = 2 * NH * kBox;
     constexpr int QW = D / 2 + 4;                     // words per query row: conflict-free fragment reads
+    constexpr int kN = kTreeParts<NTN>, kHN = kN == 3 ? 2 : NTN;
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     __shared__ __align__(8) uint64_t full[kTaStages], empty[kTaStages];
     __shared__ unsigned long long s_mask[NP];         // each pair's row mask
     uint8_t *ring = (uint8_t *)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-    uint32_t *qh = (uint32_t *)(ring + kTaStages * kStage), *ql = qh + NP * QW;  // [NP][QW] bf16 pairs
-    float *po = (float *)qh;                          // [NP][D] this rank's output, after the key loop
-    float *pm = (float *)(ql + NP * QW), *pl = pm + NP;
+    uint32_t *qp = (uint32_t *)(ring + kTaStages * kStage);   // [part][NP][QW] bf16 pairs
+    float *po = (float *)qp;                          // [NP][D] this rank's output, after the key loop
+    float *pm = (float *)(qp + kN * NP * QW), *pl = pm + NP;
     float *wo = (float *)ring;                        // [warp][NP][D], after the key loop
     float *wm = wo + W * NP * D, *wl = wm + W * NP;   // [warp][NP]
 
@@ -1211,22 +1232,25 @@ __global__ void __launch_bounds__(TaCfg<8>::kThreads, 1)
         store4(vc + 8 * q, v0.x, v0.y, v0.z, v0.w);
         store4(vc + 8 * q + 4, v1.x, v1.y, v1.z, v1.w);
     }
-    // queries, rotated, in log2 units (log2(e) / sqrt(D)), as bf16 hi + lo
-    const float scale = 1.4426950408889634f / sqrtf((float)D);
+    // queries, rotated, as bf16 parts; the scores are in log2 units (log2(e) / sqrt(D)), by a
+    // factor on the queries or, with three parts, on the scores: one rounding less
+    const float log2_scale = 1.4426950408889634f / sqrtf((float)D);
+    const float scale = kN == 3 ? 1.f : log2_scale, s_scale = kN == 3 ? log2_scale : 1.f;
     for (int e = tid; e < NP * (half / 2); e += kThr) {
         const int pr = e / (half / 2), q = e % (half / 2);
-        uint32_t h0 = 0, l0 = 0, h1 = 0, l1 = 0;
+        uint32_t w0[kN] = {}, w1[kN] = {};
         if (pr < NQ) {
             const float *x = a.qkv + (((size_t)b * a.w + pr / G) * H + g * G + pr % G) * D;
             const float2 x0 = __ldcg((const float2 *)x + q), x1 = __ldcg((const float2 *)(x + half) + q);
             const float2 c = __ldg((const float2 *)cs_row + q), s = __ldg((const float2 *)sn_row + q);
-            split2((x0.x * c.x - x1.x * s.x) * scale, (x0.y * c.y - x1.y * s.y) * scale, h0, l0);
-            split2((x1.x * c.x + x0.x * s.x) * scale, (x1.y * c.y + x0.y * s.y) * scale, h1, l1);
+            split_n<kN>((x0.x * c.x - x1.x * s.x) * scale, (x0.y * c.y - x1.y * s.y) * scale, w0);
+            split_n<kN>((x1.x * c.x + x0.x * s.x) * scale, (x1.y * c.y + x0.y * s.y) * scale, w1);
         }
-        qh[pr * QW + q] = h0;
-        ql[pr * QW + q] = l0;
-        qh[pr * QW + half / 2 + q] = h1;
-        ql[pr * QW + half / 2 + q] = l1;
+#pragma unroll
+        for (int i = 0; i < kN; ++i) {
+            qp[(i * NP + pr) * QW + q] = w0[i];
+            qp[(i * NP + pr) * QW + half / 2 + q] = w1[i];
+        }
     }
     // the async proxy reads rows this kernel just wrote: order those writes first
     asm volatile("fence.proxy.async.global;" ::: "memory");
@@ -1288,79 +1312,88 @@ __global__ void __launch_bounds__(TaCfg<8>::kThreads, 1)
                                      ::"r"(ta_piece<kC>(vb, kr + cnt + e / (NH * 8), e % (NH * 8))), "r"(0) : "memory");
                     __syncwarp();
                 }
-                float sh[NTN][4] = {}, sl[NTN][4] = {};
 #pragma unroll
-                for (int ks = 0; ks < NT; ++ks) {
-                    uint32_t ka[4];
-                    ldsm_x4(ta_piece<kC>(kb, kr + (mi & 1) * 8 + (lane & 7), 2 * ks + (mi >> 1)), ka);
+                for (int h = 0; h < NTN; h += kHN) {
+                    float sh[kHN][4] = {}, sl[kHN][4] = {};       // of the first parts, of the others
 #pragma unroll
-                    for (int nt = 0; nt < NTN; ++nt) {
-                        const int q = qo + nt * 8 * QW + 8 * ks;
-                        mma16816(sh[nt], ka, qh[q], qh[q + 4]);
-                        mma16816(sl[nt], ka, ql[q], ql[q + 4]);
+                    for (int ks = 0; ks < NT; ++ks) {
+                        uint32_t ka[4];
+                        ldsm_x4(ta_piece<kC>(kb, kr + (mi & 1) * 8 + (lane & 7), 2 * ks + (mi >> 1)), ka);
+#pragma unroll
+                        for (int u = 0; u < kHN; ++u) {
+                            if (h + u >= NTN) continue;
+                            const uint32_t *q = qp + qo + (h + u) * 8 * QW + 8 * ks;
+                            mma16816(sh[u], ka, q[0], q[4]);
+#pragma unroll
+                            for (int n = 1; n < kN; ++n) mma16816(sl[u], ka, q[n * NP * QW], q[n * NP * QW + 4]);
+                        }
                     }
-                }
-                uint32_t pbh[NTN][2], pbl[NTN][2];
+                    uint32_t pb[kHN][kN][2];
 #pragma unroll
-                for (int nt = 0; nt < NTN; ++nt) {
-                    float sv[4];
+                    for (int u = 0; u < kHN; ++u) {
+                        const int nt = h + u;
+                        if (nt >= NTN) continue;
+                        float sv[4];
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) sv[q] = sh[nt][q] + sl[nt][q];
-                    if (key0 + 16 > base || cnt < 16) {           // draft slots, or the range's end
+                        for (int q = 0; q < 4; ++q) sv[q] = (sh[u][q] + sl[u][q]) * s_scale;
+                        if (key0 + 16 > base || cnt < 16) {           // draft slots, or the range's end
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int key = (lane >> 2) + (q >> 1) * 8, off = key0 + key - base;
+                                const unsigned long long m = s_mask[nt * 8 + 2 * (lane & 3) + (q & 1)];
+                                const bool vis = key < cnt && (off < 0 || (off < kTreeMaskBits && ((m >> off) & 1ull)));
+                                if (!vis) sv[q] = -INFINITY;
+                            }
+                        }
+                        float c0 = fmaxf(sv[0], sv[2]), c1 = fmaxf(sv[1], sv[3]);
+#pragma unroll
+                        for (int off = 4; off < 32; off <<= 1) {
+                            c0 = fmaxf(c0, __shfl_xor_sync(0xFFFFFFFFu, c0, off));
+                            c1 = fmaxf(c1, __shfl_xor_sync(0xFFFFFFFFu, c1, off));
+                        }
+                        const float n0 = fmaxf(mx[nt][0], c0), n1 = fmaxf(mx[nt][1], c1);
+                        float p[4];
 #pragma unroll
                         for (int q = 0; q < 4; ++q) {
-                            const int key = (lane >> 2) + (q >> 1) * 8, off = key0 + key - base;
-                            const unsigned long long m = s_mask[nt * 8 + 2 * (lane & 3) + (q & 1)];
-                            const bool vis = key < cnt && (off < 0 || (off < kTreeMaskBits && ((m >> off) & 1ull)));
-                            if (!vis) sv[q] = -INFINITY;
+                            const float mq = (q & 1) ? n1 : n0;
+                            p[q] = (sv[q] == -INFINITY || mq == -INFINITY) ? 0.f : exp2f(sv[q] - mq);
+                        }
+                        if (__any_sync(0xFFFFFFFFu, n0 != mx[nt][0] || n1 != mx[nt][1])) {
+                            const float al0 = mx[nt][0] == -INFINITY ? 0.f : exp2f(mx[nt][0] - n0);
+                            const float al1 = mx[nt][1] == -INFINITY ? 0.f : exp2f(mx[nt][1] - n1);
+                            sm[nt][0] *= al0;
+                            sm[nt][1] *= al1;
+#pragma unroll
+                            for (int t = 0; t < NT; ++t) {
+                                o[nt][t][0] *= al0;
+                                o[nt][t][1] *= al1;
+                                o[nt][t][2] *= al0;
+                                o[nt][t][3] *= al1;
+                            }
+                        }
+                        sm[nt][0] += p[0] + p[2];
+                        sm[nt][1] += p[1] + p[3];
+                        mx[nt][0] = n0;
+                        mx[nt][1] = n1;
+                        uint32_t p01[kN], p23[kN];
+                        split_n<kN>(p[0], p[1], p01);
+                        split_n<kN>(p[2], p[3], p23);
+#pragma unroll
+                        for (int n = 0; n < kN; ++n) {
+                            pb[u][n][0] = movm_t(p01[n]);
+                            pb[u][n][1] = movm_t(p23[n]);
                         }
                     }
-                    float c0 = fmaxf(sv[0], sv[2]), c1 = fmaxf(sv[1], sv[3]);
 #pragma unroll
-                    for (int off = 4; off < 32; off <<= 1) {
-                        c0 = fmaxf(c0, __shfl_xor_sync(0xFFFFFFFFu, c0, off));
-                        c1 = fmaxf(c1, __shfl_xor_sync(0xFFFFFFFFu, c1, off));
-                    }
-                    const float n0 = fmaxf(mx[nt][0], c0), n1 = fmaxf(mx[nt][1], c1);
-                    float p[4];
+                    for (int t = 0; t < NT; ++t) {
+                        uint32_t va[4];
+                        ldsm_x4_t(ta_piece<kC>(vb, kr + (mi >> 1) * 8 + (lane & 7), 2 * t + (mi & 1)), va);
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) {
-                        const float mq = (q & 1) ? n1 : n0;
-                        p[q] = (sv[q] == -INFINITY || mq == -INFINITY) ? 0.f : exp2f(sv[q] - mq);
-                    }
-                    if (__any_sync(0xFFFFFFFFu, n0 != mx[nt][0] || n1 != mx[nt][1])) {
-                        const float al0 = mx[nt][0] == -INFINITY ? 0.f : exp2f(mx[nt][0] - n0);
-                        const float al1 = mx[nt][1] == -INFINITY ? 0.f : exp2f(mx[nt][1] - n1);
-                        sm[nt][0] *= al0;
-                        sm[nt][1] *= al1;
+                        for (int u = 0; u < kHN; ++u) {
+                            if (h + u >= NTN) continue;
 #pragma unroll
-                        for (int t = 0; t < NT; ++t) {
-                            o[nt][t][0] *= al0;
-                            o[nt][t][1] *= al1;
-                            o[nt][t][2] *= al0;
-                            o[nt][t][3] *= al1;
+                            for (int n = 0; n < kN; ++n) mma16816(o[h + u][t], va, pb[u][n][0], pb[u][n][1]);
                         }
-                    }
-                    sm[nt][0] += p[0] + p[2];
-                    sm[nt][1] += p[1] + p[3];
-                    mx[nt][0] = n0;
-                    mx[nt][1] = n1;
-                    uint32_t h01, l01, h23, l23;
-                    split2(p[0], p[1], h01, l01);
-                    split2(p[2], p[3], h23, l23);
-                    pbh[nt][0] = movm_t(h01);
-                    pbh[nt][1] = movm_t(h23);
-                    pbl[nt][0] = movm_t(l01);
-                    pbl[nt][1] = movm_t(l23);
-                }
-#pragma unroll
-                for (int t = 0; t < NT; ++t) {
-                    uint32_t va[4];
-                    ldsm_x4_t(ta_piece<kC>(vb, kr + (mi >> 1) * 8 + (lane & 7), 2 * t + (mi & 1)), va);
-#pragma unroll
-                    for (int nt = 0; nt < NTN; ++nt) {
-                        mma16816(o[nt][t], va, pbh[nt][0], pbh[nt][1]);
-                        mma16816(o[nt][t], va, pbl[nt][0], pbl[nt][1]);
                     }
                 }
                 // zeros written above precede the next TMA write of this slot
@@ -1452,7 +1485,7 @@ __global__ void __launch_bounds__(TaCfg<8>::kThreads, 1)
 
 template <int D, int NTN>
 constexpr size_t tree_cl_smem() {
-    return 1024 + (size_t)kTaStages * 2 * (D / 64) * TaCfg<8>::kC * 128 + (size_t)2 * 8 * NTN * (D / 2 + 4) * 4 +
+    return 1024 + (size_t)kTaStages * 2 * (D / 64) * TaCfg<8>::kC * 128 + (size_t)kTreeParts<NTN> * 8 * NTN * (D / 2 + 4) * 4 +
            (size_t)2 * 8 * NTN * 4;
 }
 static_assert((size_t)(8 * 32 * 128 + 2 * 8 * 32) * 4 <= (size_t)kTaStages * 2 * 2 * TaCfg<8>::kC * 128 &&

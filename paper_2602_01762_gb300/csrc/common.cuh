@@ -603,8 +603,8 @@ int gemv_lm_slots(const GemvArgs &a, int sms, bool streamed);
 size_t gemv_tcs_workspace_floats(const GemvArgs &a, int sms);
 // *next_done (may be null) reports whether the launch also wrote the next
 // projection's rows (a.next_norm or a.next_fuse) into a.next_x.
-cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, float *part, int *tile_ctr,
-                            uint16_t *xbuf, cudaStream_t s, bool pdl, bool *next_done = nullptr);
+cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, float *part, uint16_t *xbuf,
+                            cudaStream_t s, bool pdl, bool *next_done = nullptr);
 cudaError_t prepare_attention_kernel(bool bf16, int D, int chunk, int G, int splits);
 // Sets kernel attributes and fills *cl; `need`: the KV heads of one sequence.
 cudaError_t prepare_fused_attention(bool bf16, int D, int G, int need, AttnClusters *cl);

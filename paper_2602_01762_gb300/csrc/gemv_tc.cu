@@ -1902,17 +1902,16 @@ cudaError_t launch_topk_merge(const GemvArgs &a, int slots, cudaStream_t s) {
     return launch_k(topk_merge_kernel, dim3(a.T), dim3(128), 0, s, true, a, slots);
 }
 
-cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, float *part, int *tile_ctr,
-                            uint16_t *xbuf, cudaStream_t s, bool pdl, bool *next_done) {
+cudaError_t launch_gemv_tcs(const GemvArgs &a, const CUtensorMap &mw, int sms, float *part, uint16_t *xbuf,
+                            cudaStream_t s, bool pdl, bool *next_done) {
     if (next_done) *next_done = false;
     TcPlan p{};
     int grid, NB;
     size_t smem;
     if (!tcs_plan(a, sms, p, grid, smem, NB)) return cudaErrorInvalidValue;
     p.part = part;
-    p.tile_ctr = tile_ctr;
     p.defer = p.splits > 1;
-    if (p.splits > 1 && (!part || !tile_ctr)) return cudaErrorInvalidValue;
+    if (p.splits > 1 && !part) return cudaErrorInvalidValue;
     // the activation rows as a bf16 [T][kin] buffer: the copy prologue's
     // source as it is, otherwise written by prep_x_kernel
     const void *x = a.act;

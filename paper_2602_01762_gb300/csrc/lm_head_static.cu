@@ -127,7 +127,7 @@ cudaError_t launch_streamed(GemvArgs g, const CUtensorMap &tm, int r0, int rows,
     const size_t lists = (size_t)rows * slots * kTopK * 8;
     uint16_t *x = (uint16_t *)(st.scratch + kHeadBytes + ((lists + 255) & ~(size_t)255));
     g.best = rows <= kTop1Rows ? (unsigned long long *)(st.scratch + 128) : nullptr;
-    return launch_gemv_tcs(g, tm, st.sms, nullptr, nullptr, x, s, false);
+    return launch_gemv_tcs(g, tm, st.sms, nullptr, x, s, false);
 }
 
 }  // namespace

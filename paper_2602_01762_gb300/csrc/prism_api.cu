@@ -279,8 +279,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
         if (!(tm && want_tc(g) && c->tc_ready && c->bf16 && (g.T >= rows_min || lm1) &&
               gemv_tcs_supported(g, c->sms)))
             return false;
-        const size_t ws = gemv_tcs_workspace_floats(g, c->sms);
-        return ws == 0 || (ws <= c->tc_part_floats && gemv_tc_tiles(g) <= c->tc_ctr_n);
+        return gemv_tcs_workspace_floats(g, c->sms) <= c->tc_part_floats;
     };
     // the staged tcgen05 kernel takes g (when the streamed one does not)
     auto on_tc_staged = [&](const GemvArgs &g, const CUtensorMap *tm) -> bool {
@@ -314,7 +313,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
                 }
             }
             bool done = false;
-            const cudaError_t le = launch_gemv_tcs(g, *tm, c->sms, c->tc_part, c->tc_ctr, c->xbuf, s, pdl_here, &done);
+            const cudaError_t le = launch_gemv_tcs(g, *tm, c->sms, c->tc_part, c->xbuf, s, pdl_here, &done);
             x_ready = le == cudaSuccess && done;
             return le;
         }

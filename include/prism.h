@@ -135,6 +135,9 @@ prism_status prism_load_step_weights(prism_ctx *ctx, int32_t step, const prism_s
  *   logits      float [batch, K, V]           out, or NULL
  *   hidden_out  float [batch, K, d]           out (h^_0 .. h^_{K-1}), or NULL
  * Ties in the argmax go to the lowest id; top-k is sorted by logit, then id.
+ * A NaN logit is no candidate; a place for which there is none holds id
+ * 0x7FFFFFFF and logit -inf (as a drafted token it sets the token bit of the
+ * device error word at the next step).
  * The round is captured once per distinct argument set as a CUDA graph and
  * replayed (option "use_graph").  Errors: INVALID_ARG, CAPACITY
  * (batch > max_batch), NOT_LOADED, CUDA. */
@@ -271,7 +274,7 @@ typedef struct {
  *     the next frontier is the w best of the w^2 new candidates;
  *   end: the verified tree is the n_nodes best candidates of the round.
  * Orders: top-w by logit, then id; frontiers and the tree by score
- * descending, then pool index ascending.
+ * descending (NaN as -inf), then pool index ascending.
  *   width        1..max_tree_width; (K - 1) * width <= 64; P <= 1024
  *   n_nodes      1..P
  *   out          see prism_tree_outputs (tokens, parents, depths, scores
@@ -311,16 +314,20 @@ prism_status prism_accept_tree(prism_ctx *ctx, int32_t batch, int32_t n_nodes, c
  * framework forbids allocation outside its own pool, or a process that fixes
  * its whole device-memory budget at start-up.
  * It computes what the last stage of a draft step computes (final RMSNorm with
- * gain g_final, logits = lm_head . norm(h), top-1 and top-k), using the same
- * kernel, and keeps that kernel's scratch (the per-CTA partial top-8 lists,
- * the last-CTA ticket and the device error word) in a static device array of
- * 1 MiB + 256 bytes inside the library, which every process that loads the
- * library holds on each device it uses until exit.
+ * gain g_final, logits = lm_head . norm(h), top-1 and top-k), with the same
+ * kernels, and keeps their scratch (the per-CTA partial top-8 lists, bf16
+ * activation rows, packed top-1 keys, the last-CTA ticket and the device error
+ * word) in a static device array of 1 MiB + 256 bytes inside the library, which
+ * every process that loads the library holds on each device it uses until
+ * exit.  With PRISM_BF16 a pass over the weights takes as many rows as that
+ * array holds (64 of hidden 1024, 58 of 4096, 40 of 8192 on 152 SMs), the rest
+ * go in further passes.
  *   dtype PRISM_F32 or PRISM_BF16 (the type of lm_head and g_final);
  *   h fp32 [batch, hidden] hidden rows before the final norm;
  *   g_final [hidden] or NULL (no final norm); lm_head [vocab, hidden];
  *   draft int32 [batch] out; topk_ids int32 [batch, topk], topk_logits fp32
- *   [batch, topk], logits fp32 [batch, vocab]: outputs, each may be NULL;
+ *   [batch, topk], logits fp32 [batch, vocab]: outputs, each of these three may
+ *   be NULL (places without a candidate as in prism_draft_round);
  *   dev_flags int32 [1] or NULL: receives the device error word of this call.
  * All pointers are device (or managed) memory of the current device; h,
  * lm_head and g_final 16-byte aligned.  A pointer to host memory or to
@@ -329,9 +336,9 @@ prism_status prism_accept_tree(prism_ctx *ctx, int32_t batch, int32_t n_nodes, c
  * message from prism_get_error(NULL): split them into several calls.
  * The first call on a device (the current one) does that device's set-up:
  * it resolves the array's device address with cudaGetSymbolAddress and sets
- * the kernel's shared-memory attribute; make that first call before any
- * stream capture.  Each call clears the ticket and the error word with a
- * stream-ordered memset, then launches the kernel on `stream`.  Every call
+ * the kernels' shared-memory attributes; make that first call before any
+ * stream capture.  Each call clears the ticket, the keys and the error word with
+ * a stream-ordered memset, then launches its kernels on `stream`.  Every call
  * shares the one array, so calls that can overlap on the GPU (different
  * streams, or several host threads) race and corrupt each other's results:
  * keep them on one stream.  Calls no cudaMalloc, cudaFree or allocating
@@ -353,13 +360,13 @@ prism_status prism_sync_status(prism_ctx *ctx, void *stream, int32_t *flags);
 
 /* Options (name, value): "use_graph" (1: capture and replay, default 1),
  * "use_pdl" (1: programmatic dependent launch between kernels, default 1),
- * "gemv_chunk_kb" (target TMA stage size of the projection kernels, 0..128,
- * 0 = default), "gemv_smem_kb" (shared-memory budget of the projection
- * ring, 0..200, 0 = default), "gemv_groups" (consumer warp groups of the
- * projection kernels: 1, 2, 4, 8 or 16; 0 = default), "gemv_tcgen05"
+ * "gemv_chunk_kb" (target TMA stage size of the bf16 CUDA-core projection
+ * kernel, 0..128, 0 = default), "gemv_smem_kb" (shared-memory budget of its
+ * ring, 0..200, 0 = default), "gemv_groups" (its consumer warp groups: 1, 2, 4,
+ * 8 or 16; 0 = default), "gemv_tcgen05"
  * (1, the default: bf16 projections run on the tcgen05 kernels, TMA tensor
- * loads into tensor-memory accumulators, except gate/up + SwiGLU with at
- * most 2 activation rows, which measures faster on the CUDA-core kernel;
+ * loads into tensor-memory accumulators, except gate/up + SwiGLU with one
+ * activation row, which measures faster on the CUDA cores;
  * 2: gate/up as well; 0: every projection on the kernels below),
  * "tc_stream_rows" (>= 1, default 1: a tcgen05 projection with at least
  * this many activation rows streams them through the TMA ring beside the

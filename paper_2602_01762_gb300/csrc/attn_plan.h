@@ -26,7 +26,7 @@ struct AttnPlan {
 // cache rows beyond which two-CTA clusters keep 8 warps.  Both look at the cache's
 // capacity: the contexts are device data that the host does not know at a launch.
 constexpr long long kAttnSmallCache = 8LL << 20;
-constexpr int kAttnLongCtx = 3072;
+constexpr int kAttnLongCtx = 3072;   // see attn_plan
 
 inline bool attn_small_cache(const AttnSizes &z) { return z.cache_bytes < kAttnSmallCache; }
 
@@ -60,9 +60,13 @@ inline AttnPlan attn_plan(const AttnClusters &cl, const AttnSizes &z, int want_w
     // 64: 2050 us a round with 8 warps, 2009 with 4; 7B shape, batch 16, 1937
     // and 1875).  Clusters of two in two waves over long caches keep 8 warps:
     // twice the bytes in flight per CTA and, with the longest sequences first,
-    // a short tail (8B shape, contexts 512 to 4096, batch 12: 1430 us with 8,
-    // 1472 with 4; contexts 512 to 2000: 1413 and 1406).  Small caches: one wave
-    // of single CTAs only (as for their clusters)
+    // a short tail where the contexts are uneven.  8B shape, 3 steps, batch 10 / 16, us
+    // a round with 8 warps and with 4: contexts 512 to 2048 822 / 885 and 818 / 869, to
+    // 3040 824 / 892 and 831 / 888, to 4096 846 / 902 and 850 / 906, to 8000 863 / 955 and
+    // 909 / 982 (7B shape, batch 3, 535 and 568).  Even contexts would take 4 warps at any
+    // length (4096: 912 / 960 and 861 / 938), and so would short ones in a long cache
+    // (512 to 2048 of 16384: 819 / 885 and 820 / 870), which a launch cannot tell.
+    // Small caches: one wave of single CTAs only (as for their clusters)
     const long long n_ctas = (long long)z.B * z.Hkv * p.cs;
     const bool long_pairs = p.cs == 2 && z.B > 1 && z.max_ctx > kAttnLongCtx;
     const bool four = p.cs <= 8 && (attn_small_cache(z) ? p.cs == 1 && n_ctas <= 2LL * z.sms : !long_pairs);

@@ -21,7 +21,8 @@
 //     take 8 rows each of the same item.
 //   * Small layers run as 8-warp CTAs of at most 110 KB, two to an SM, so that
 //     the next projection's CTAs start and fill their rings while this one's
-//     drain; layers with more bytes per SM as 16-warp CTAs with a larger ring.
+//     drain; layers with more bytes per SM as 16-warp CTAs with a larger ring
+//     (small_layer has what either is worth).
 //   * The LM head keeps the CTA's logits in shared memory, selects once per
 //     chunk of units, publishes one list per row, and topk_merge_kernel joins
 //     the CTAs' lists (the last CTA did that alone, with dependent loads).
@@ -410,7 +411,17 @@ cudaError_t f32_attrs() {
     return e;
 }
 
-// A layer with fewer bytes per CTA than this runs as 8-warp CTAs, two to an SM.
+// A layer with fewer bytes per CTA than this runs as 8-warp CTAs, two to an SM, and
+// makes no L2 requests for the next; a bf16 gate/up row of such a layer stays on the
+// ring kernel.  The line was drawn between hidden 1024 (up to 160 KB per CTA outside the
+// LM head) and 4096 (450 KB and more).  Both sides of it since (K 4, vocabulary
+// 32000, contexts of 200, us a round; every layer as 16-warp CTAs in brackets), fp32 rounds of
+// 1 / 3 / 12 sequences: hidden 256 161 / 184 / 377 (170 / 172 / 284), 1024 256 / 320 / 620
+// (252 / 296 / 539), 2048 443 / 540 / 1141 (421 / 494 / 1048), 3072 685 / 842 / 2046 (675 /
+// 822 / 2022), 4096 the same: the 8-warp CTAs pay for one sequence at hidden 256 alone.
+// One bf16 sequence on the ring kernel and on this one: hidden 1024 201 and 195 us, 1536 233
+// and 232, 2048 with 304 KB per CTA 287 and 283, with 432 KB 307 and 299, 3072 397 and 390,
+// 4096 562 and 560: nowhere a loss since small layers' L2 requests went (198 and 207 before).
 bool small_layer(const GemvArgs &a, int es, int grid) {
     const int UI = a.epi == kEpiSwiGLU ? kMR / 2 : kMR;
     const int n_items = (a.n_units + UI - 1) / UI, per_cta = (n_items + grid - 1) / grid;
@@ -424,7 +435,8 @@ bool f32_plan(const GemvArgs &a, int es, int grid, F32Plan &p, size_t &smem) {
     const int n_items = (a.n_units + UI - 1) / UI, per_cta = (n_items + grid - 1) / grid;
     const bool small = small_layer(a, es, grid);
     // beside such CTAs the next layer's own rings are already filling: requests
-    // for its first bytes only delay them (339 us a round with, 327 without, three sequences as above)
+    // for its first bytes only delay them (three sequences at hidden 1024, on the build
+    // of that step: 339 us a round with, 327 without)
     p.prefetch = !small;
     p.tn = a.T <= 1 ? 1 : a.T <= 2 ? 2 : a.T <= 4 ? 4 : 8;
     p.tg = a.T <= 8 ? 1 : a.T <= 16 ? 2 : 4;
@@ -469,8 +481,7 @@ cudaError_t prepare_gemv_f32_kernels() {
 bool gemv_pair_supported(const GemvArgs &a, int grid) {
     F32Plan p{};
     size_t smem;
-    // (a small layer stays on the ring kernel, which norms its row itself: hidden
-    // 1024, batch 1, 198 us a round there and 207 here)
+    // (a small layer stays on the ring kernel, which norms its row itself; see small_layer)
     return a.epi == kEpiSwiGLU && a.T == 1 && !small_layer(a, 2, grid) && f32_plan(a, 2, grid, p, smem);
 }
 

@@ -10,7 +10,8 @@
 // Llama-3-8B vocabulary (1.05 GB) take 170 us a call, 6.2 TB/s, against 1104 us
 // on the CUDA-core ring, which reads every row from shared memory once per
 // weight row.
-// fp32, and shapes the streamed kernel does not take, stay on that ring.
+// fp32 runs on gemv_rows4_kernel and the merge kernel; bf16 shapes that the streamed
+// kernel does not take, on that ring.
 //
 // Some callers cannot call cudaMalloc: an inference server whose caching
 // allocator has already reserved the device memory it may use, a plugin whose

@@ -264,8 +264,7 @@ cudaError_t enqueue_round(prism_ctx *c, const RoundArgs &r, cudaStream_t s, bool
     };
     // the streamed tcgen05 kernel takes g (its activation rows in the bf16 buffer)
     auto on_tcs = [&](const GemvArgs &g, const CUtensorMap *tm) -> bool {
-        // the top-1 LM head streams its rows from one row on with lm_stream
-        // (not in sampled rounds, whose draw reads the logits it writes)
+        // a greedy round's top-1 LM head streams its rows from one row on with lm_stream
         const bool lm1 = c->lm_stream && g.stream_top1 && g.epi == kEpiTopK && g.topk == 1 && g.best;
         // any other greedy LM head (top-k lists; lm_stream off) keeps fewer than
         // 8 rows staged, where its lists merge without another kernel; a sampled
